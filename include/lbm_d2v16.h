@@ -301,7 +301,7 @@ int lbm_fault_inject(lbm_handle h, int what, long long wait_cycles);
  * energy agrees to about 1e-6 (relative), the other values to about 1e-12.
  * It calls no cudaMalloc, cudaFree or allocating library routine: its scratch (d_x rho,
  * d_y rho, per-block partial sums, derivative tables) is one file-scope device array of
- * about 16.3 MiB, which every GPU that loads this library holds until the process exits; its
+ * about 16.2 MiB, which every GPU that loads this library holds until the process exits; its
  * device address is looked up (cudaGetSymbolAddress) on every call, in the current device's
  * context. Limits: nx, ny powers of two in [2, 4096] and nx * ny <= 1048576 (e.g. 1024 x 1024);
  * larger sizes return LBM_ERR_ARG with the reason in lbm_last_error(). Work is issued on

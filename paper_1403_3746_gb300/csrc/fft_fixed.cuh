@@ -1,0 +1,217 @@
+// 64-bit fixed-point arithmetic for the float64 line transforms (Sec. 2.3 / Eq. (3)).
+//
+// GB300 issues 2 float64 operations per clock and SM, but 128 32-bit integer additions and 64
+// 32-bit multiply-adds (measured: add.s64 64 per clock and SM, mul.wide.s32 60, fma.f64 2.0). A
+// complex butterfly addition is four integer instructions instead of two float64 ones that take
+// 32 times their slots, so the float64 lines are transformed as 64-bit integers that share one
+// exponent per complex line (block floating point).
+//
+// Scaling of a line of N = 2^LOG2N points. Let 2^e bound the magnitude of the line's 2 N real
+// numbers (from their exponents). Point x enters as round(x 2^(B - e)), |Re|, |Im| < 2^B. Every
+// radix-16 pass that has outer twiddles ends (forward) or begins (inverse) with a factor 1/4,
+// which the high half of the product with a root scaled to 2^62 gives for free. B is the largest
+// value for which a sum of moduli cannot reach 2^63 anywhere in the forward passes: moduli start
+// below 2^(B + 1/2), a radix-16 pass multiplies them by at most 16, so B = 62 - (largest growth).
+// The spectrum's 2-norm is at most N 2^(B + 1/2) / 4^T (T twiddled passes); the multiplier,
+// normalised to at most 1, is applied with another factor 1/4, and a sum of P of its points is at
+// most sqrt(P) times the 2-norm (Cauchy-Schwarz), which stays below 2^63 in every inverse pass for
+// every LOG2N <= 12. So no line can overflow, whatever its values.
+//
+// Rounding: each product is rounded to the nearest integer up to a quarter unit, inputs are
+// rounded once at 2^(e - B) (B = 54 .. 58), and before the inverse the spectrum is shifted up as
+// far as the sum of its magnitudes allows. Error of a derivative against __float128 sums, relative
+// to the float64 transform's, 8 .. 4096 points: 0.1 to 0.8 for lines with a mean, smooth, noisy or
+// step-like ones and for peaks a few points wide (1.06 for those at 4096), 1.8 to 2.8 for lines that
+// are zero but for one point (8e-16 of the result at most).
+//
+// Measured against the float64 transforms (1024^2, float64 step): column pass 1230 -> 524 us per
+// launch of 17 fields, flux pass 332 -> 160, step 8.31 -> 5.46 ms.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace lbm {
+namespace fixed {
+
+template <typename R> struct is_fixed {
+    static constexpr bool value = false;
+};
+template <> struct is_fixed<long long> {
+    static constexpr bool value = true;
+};
+
+// Second factors (roots, multipliers) are stored as balanced halves: low 32 bits as a signed
+// integer bl in [-2^31, 2^31), high 32 bits bh with b = bh 2^32 + bl, |b| <= 2^63 - 2^31.
+__host__ __device__ __forceinline__ long long balance(long long b) {
+    return (long long)(((unsigned long long)(b + 0x80000000LL) & 0xffffffff00000000ULL) |
+                       ((unsigned long long)b & 0xffffffffULL));
+}
+__host__ __device__ __forceinline__ int lo32(long long a) { return (int)(unsigned)(unsigned long long)a; }
+__host__ __device__ __forceinline__ int hi32(long long a) { return (int)(a >> 32); }
+// high half of a in balanced halves
+__host__ __device__ __forceinline__ int bal_hi(long long a) {
+    return hi32(a) + (int)((unsigned)lo32(a) >> 31);
+}
+
+// a b / 2^64 to the nearest integer (error at most 3/4: the low halves' product is left out),
+// a as balanced halves (ah, al), b as (bh, bl); |a| <= 2^62.5
+__host__ __device__ __forceinline__ long long mulhi(int ah, int al, int bh, int bl) {
+    const long long m = (long long)ah * bl + ((long long)al * bh + 0x80000000LL);
+    return (long long)ah * bh + (m >> 32);
+}
+__host__ __device__ __forceinline__ long long mulhi(long long a, long long b_balanced) {
+    return mulhi(bal_hi(a), lo32(a), hi32(b_balanced), lo32(b_balanced));
+}
+
+__host__ __device__ __forceinline__ longlong2 mk2(long long x, long long y) {
+    longlong2 c;
+    c.x = x;
+    c.y = y;
+    return c;
+}
+// a / 4, rounded
+__host__ __device__ __forceinline__ longlong2 quarter(longlong2 a) { return mk2((a.x + 2) >> 2, (a.y + 2) >> 2); }
+
+// a w / 4 and a conj(w) / 4, w scaled to 2^62 in balanced halves
+__host__ __device__ __forceinline__ longlong2 mul4(longlong2 a, longlong2 w) {
+    const int xh = bal_hi(a.x), xl = lo32(a.x), yh = bal_hi(a.y), yl = lo32(a.y);
+    const int ch = hi32(w.x), cl = lo32(w.x), sh = hi32(w.y), sl = lo32(w.y);
+    return mk2(mulhi(xh, xl, ch, cl) - mulhi(yh, yl, sh, sl), mulhi(xh, xl, sh, sl) + mulhi(yh, yl, ch, cl));
+}
+__host__ __device__ __forceinline__ longlong2 mulc4(longlong2 a, longlong2 w) {
+    const int xh = bal_hi(a.x), xl = lo32(a.x), yh = bal_hi(a.y), yl = lo32(a.y);
+    const int ch = hi32(w.x), cl = lo32(w.x), sh = hi32(w.y), sl = lo32(w.y);
+    return mk2(mulhi(xh, xl, ch, cl) + mulhi(yh, yl, sh, sl), mulhi(yh, yl, ch, cl) - mulhi(xh, xl, sh, sl));
+}
+
+// Constants of the 16-point transform, scaled to 2^64 (all below 1/2): tan(pi/16), sin(pi/8),
+// 1 - sqrt(1/2)
+constexpr unsigned long long kTan = 0x32EBEBC0AA62B00FULL;
+constexpr unsigned long long kSin = 0x61F78A9ABAA58B47ULL;
+constexpr unsigned long long kOneMinusSqrtHalf = 0x4AFB0CCC06219B7CULL;
+
+// a (constant c / 2^64)
+template <unsigned long long C> __host__ __device__ __forceinline__ long long scale_const(long long a) {
+    constexpr int bl = (int)(unsigned)(C & 0xffffffffULL);
+    constexpr int bh = (int)((C + 0x80000000ULL) >> 32);
+    return mulhi(bal_hi(a), lo32(a), bh, bl);
+}
+// rotation by -pi/8 (NEG) or +pi/8 as three shears (lifting steps): three products instead of four
+template <bool NEG> __host__ __device__ __forceinline__ longlong2 rot_pi8(longlong2 a) {
+    const long long d = scale_const<kTan>(a.y);
+    const long long x = NEG ? a.x + d : a.x - d;
+    const long long g = scale_const<kSin>(x);
+    const long long y = NEG ? a.y - g : a.y + g;
+    const long long h = scale_const<kTan>(y);
+    return mk2(NEG ? x + h : x - h, y);
+}
+__host__ __device__ __forceinline__ long long sqrt_half(long long a) {
+    return a - scale_const<kOneMinusSqrtHalf>(a);
+}
+// a w16^M, unscaled (w16 = exp(-2 pi i / 16), the conjugate if INV)
+template <bool INV, int M> __host__ __device__ __forceinline__ longlong2 w16(longlong2 a) {
+    static_assert(M == 1 || M == 2 || M == 3 || M == 4 || M == 6 || M == 9, "roots of the 16-point transform");
+    // multiplication by w16^4 = -i (forward), +i (inverse)
+    auto quarter_turn = [](longlong2 z) { return INV ? mk2(-z.y, z.x) : mk2(z.y, -z.x); };
+    if constexpr (M == 1) return rot_pi8<!INV>(a);
+    if constexpr (M == 2) {
+        return INV ? mk2(sqrt_half(a.x - a.y), sqrt_half(a.x + a.y)) : mk2(sqrt_half(a.x + a.y), sqrt_half(a.y - a.x));
+    }
+    if constexpr (M == 3) return quarter_turn(rot_pi8<INV>(a));
+    if constexpr (M == 4) return quarter_turn(a);
+    if constexpr (M == 6) {
+        const long long s = sqrt_half(a.x + a.y), d = sqrt_half(a.y - a.x);
+        return INV ? mk2(-s, -d) : mk2(d, -s);
+    }
+    if constexpr (M == 9) {
+        const longlong2 r = rot_pi8<!INV>(a);
+        return mk2(-r.x, -r.y);
+    }
+}
+
+// ---- line scaling ------------------------------------------------------------------------
+constexpr int kMaxBits = 58;  // a first radix-16 pass multiplies moduli by up to 16
+// bits of an input point (see above): 62 minus the largest growth of the forward passes
+__host__ __device__ constexpr int input_bits(int log2n) {
+    int g = 0, top = 0, left = log2n;
+    if (log2n >= 4)
+        while (left >= 4) {
+            g += 4;
+            top = g > top ? g : top;
+            left -= 4;
+            if (left > 0) g -= 2;  // a twiddled pass
+        }
+    g += left;
+    top = g > top ? g : top;
+    return 62 - top < kMaxBits ? 62 - top : kMaxBits;
+}
+
+// exponent fields below this (2^-959) count as zero, a line of such values transforms to zero
+constexpr int kMinExp = 64;
+
+// input bits of a line whose sum of |Re| + |Im| is at most 2^c 2^e: a sum of moduli never exceeds
+// 2^c, so sparse lines (fluxes that live on an interface) get more bits than the bound by the maximum
+// alone allows
+template <int LOG2N> __host__ __device__ __forceinline__ int line_bits(int c) {
+    constexpr int base = input_bits(LOG2N);
+    const int b = 62 - c < kMaxBits ? 62 - c : kMaxBits;
+    return b > base ? b : base;
+}
+
+// round(x 2^(B - e)) from the bits of the double x; e = emax - 1022 (emax: the largest exponent
+// field of the line, kMinExp <= emax <= 2046), top = emax + kMaxBits - B
+__host__ __device__ __forceinline__ long long from_double(unsigned long long x, int top) {
+    const int hi = (int)(x >> 32);
+    int d = top - (int)(((unsigned)hi >> 20) & 0x7ffu);
+    d = d < 63 ? d : 63;
+    const unsigned long long mant =
+        ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | (x & 0xffffffffULL);
+    const long long v = (long long)((((mant << (kMaxBits - 52)) >> d) + 1) >> 1);
+    return hi < 0 ? -v : v;
+}
+// |x| as a float from the high word of its bits, truncated; 0 below the float's normal range,
+// not meaningful above it
+__host__ __device__ __forceinline__ float abs_approx(unsigned long long x) {
+    const int h = (int)((x >> 32) & 0x7fffffffu) - (896 << 20);
+    const unsigned b = h > 0 ? (unsigned)h << 3 : 0u;
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(b);
+#else
+    float f;
+    __builtin_memcpy(&f, &b, 4);
+    return f;
+#endif
+}
+
+__host__ __device__ __forceinline__ int clz64(unsigned long long m) {
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)m);
+#else
+    return m ? __builtin_clzll(m) : 64;
+#endif
+}
+// bits of the double y 2^ex, rounded to nearest, -960 <= ex <= 950 (no overflow or underflow)
+__host__ __device__ __forceinline__ unsigned long long to_double(long long y, int ex) {
+    const unsigned long long m = y < 0 ? 0ULL - (unsigned long long)y : (unsigned long long)y;
+    const int lz = clz64(m);
+    const unsigned long long v = (((m << lz) >> 10) + 1) >> 1;  // in [2^52, 2^53]
+    const unsigned hi = (unsigned)(v >> 32) + ((unsigned)(ex + 1023 + 62 - lz) << 20);
+    const unsigned long long r = ((unsigned long long)(hi | ((unsigned)(y >> 32) & 0x80000000u)) << 32) | (v & 0xffffffffULL);
+    return m ? r : 0ULL;
+}
+
+// A real factor c = m 2^ex as a fixed-point number m 2^62 (|m| in [1/2, 1)) in balanced halves
+struct Factor {
+    long long m;
+    int ex;
+};
+__host__ __device__ __forceinline__ Factor factor(unsigned long long bits) {
+    Factor f;
+    const int E = (int)((bits >> 52) & 0x7ff);
+    const long long v = (long long)(((bits & 0xfffffffffffffULL) | 0x10000000000000ULL) << 9);  // [2^61, 2^62)
+    f.m = E == 0 ? 0 : balance((long long)bits < 0 ? -v : v);
+    f.ex = E - 1022;
+    return f;
+}
+
+}  // namespace fixed
+}  // namespace lbm

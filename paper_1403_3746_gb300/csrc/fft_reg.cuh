@@ -17,20 +17,27 @@
 // conjugate roots: it takes the digit-reversed spectrum back to natural order, thread t
 // holding points t + G e (e < E), the layout in which the forward transform reads its input.
 // So rows are read and written with coalesced accesses straight from and to global memory.
+//
+// The same passes run on 64-bit fixed-point points (R = long long): fft_fixed.cuh.
 #pragma once
 #include <cuda_runtime.h>
+#include <stdint.h>
 
 namespace lbm {
 
 template <typename R> struct cplx;
 template <> struct cplx<double> { typedef double2 T; };
 template <> struct cplx<float> { typedef float2 T; };
+template <> struct cplx<long long> { typedef longlong2 T; };
 
+}  // namespace lbm
+#include "fft_fixed.cuh"
+namespace lbm {
 namespace reg {
 
 template <typename R> using C = typename cplx<R>::T;
 
-template <typename R> __device__ __forceinline__ C<R> mk(R x, R y) {
+template <typename R> __host__ __device__ __forceinline__ C<R> mk(R x, R y) {
     C<R> c;
     c.x = x;
     c.y = y;
@@ -40,33 +47,39 @@ template <typename R> __device__ __forceinline__ C<R> mk(R x, R y) {
 // two-lane instruction (add.rn.f32x2, sm_100 and later), the same IEEE results with half
 // the instructions; used by the kernels whose registers allow the pairing.
 template <typename R, bool PK> struct Arith {
-    static __device__ __forceinline__ C<R> add(C<R> a, C<R> b) { return mk<R>(a.x + b.x, a.y + b.y); }
-    static __device__ __forceinline__ C<R> sub(C<R> a, C<R> b) { return mk<R>(a.x - b.x, a.y - b.y); }
+    static __host__ __device__ __forceinline__ C<R> add(C<R> a, C<R> b) { return mk<R>(a.x + b.x, a.y + b.y); }
+    static __host__ __device__ __forceinline__ C<R> sub(C<R> a, C<R> b) { return mk<R>(a.x - b.x, a.y - b.y); }
 };
 template <> struct Arith<float, true> {
     static __device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
     static __device__ __forceinline__ float2 sub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 };
-// a * w and a * conj(w)
-template <typename R> __device__ __forceinline__ C<R> mul(C<R> a, C<R> w) {
+// a * w and a * conj(w) (fixed-point points: a quarter of it, fft_fixed.cuh)
+template <typename R> __host__ __device__ __forceinline__ C<R> mul(C<R> a, C<R> w) {
     return mk<R>(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
 }
-template <typename R> __device__ __forceinline__ C<R> mulc(C<R> a, C<R> w) {
+template <typename R> __host__ __device__ __forceinline__ C<R> mulc(C<R> a, C<R> w) {
     return mk<R>(a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y);
 }
+template <> __host__ __device__ __forceinline__ longlong2 mul<long long>(longlong2 a, longlong2 w) {
+    return fixed::mul4(a, w);
+}
+template <> __host__ __device__ __forceinline__ longlong2 mulc<long long>(longlong2 a, longlong2 w) {
+    return fixed::mulc4(a, w);
+}
 // multiplication by -i (forward) or +i (inverse)
-template <typename R, bool INV> __device__ __forceinline__ C<R> rot(C<R> a) {
+template <typename R, bool INV> __host__ __device__ __forceinline__ C<R> rot(C<R> a) {
     return INV ? mk<R>(-a.y, a.x) : mk<R>(a.y, -a.x);
 }
 
-template <typename R, bool INV, bool PK> __device__ __forceinline__ void dft2(C<R> &x0, C<R> &x1) {
+template <typename R, bool INV, bool PK> __host__ __device__ __forceinline__ void dft2(C<R> &x0, C<R> &x1) {
     const C<R> t = x0;
     x0 = Arith<R, PK>::add(t, x1);
     x1 = Arith<R, PK>::sub(t, x1);
 }
 
 // y_k = sum_q x_q w4^{qk}, w4 = exp(-+ 2 pi i / 4); in place, outputs in natural order
-template <typename R, bool INV, bool PK> __device__ __forceinline__ void dft4(C<R> &x0, C<R> &x1, C<R> &x2, C<R> &x3) {
+template <typename R, bool INV, bool PK> __host__ __device__ __forceinline__ void dft4(C<R> &x0, C<R> &x1, C<R> &x2, C<R> &x3) {
     const C<R> t0 = Arith<R, PK>::add(x0, x2), t1 = Arith<R, PK>::sub(x0, x2), t2 = Arith<R, PK>::add(x1, x3);
     const C<R> t3 = rot<R, INV>(Arith<R, PK>::sub(x1, x3));
     x0 = Arith<R, PK>::add(t0, t2);
@@ -76,27 +89,31 @@ template <typename R, bool INV, bool PK> __device__ __forceinline__ void dft4(C<
 }
 
 // a * w16^M (forward: w16 = exp(-2 pi i/16); inverse: the conjugate), M a compile-time constant
-template <typename R, bool INV, int M> __device__ __forceinline__ C<R> w16(C<R> a) {
+template <typename R, bool INV, int M> __host__ __device__ __forceinline__ C<R> w16(C<R> a) {
     constexpr int m = M & 15;
-    if (m == 0) return a;
-    if (m == 4) return rot<R, INV>(a);
-    if (m == 8) return mk<R>(-a.x, -a.y);
-    if (m == 12) return rot<R, !INV>(a);
-    // cos and sin of 2 pi m / 16
-    constexpr double cs[16] = {1.0, 0.92387953251128675613, 0.70710678118654752440, 0.38268343236508977173,
-                               0.0, -0.38268343236508977173, -0.70710678118654752440, -0.92387953251128675613,
-                               -1.0, -0.92387953251128675613, -0.70710678118654752440, -0.38268343236508977173,
-                               0.0, 0.38268343236508977173, 0.70710678118654752440, 0.92387953251128675613};
-    constexpr double sn[16] = {0.0, 0.38268343236508977173, 0.70710678118654752440, 0.92387953251128675613,
-                               1.0, 0.92387953251128675613, 0.70710678118654752440, 0.38268343236508977173,
-                               0.0, -0.38268343236508977173, -0.70710678118654752440, -0.92387953251128675613,
-                               -1.0, -0.92387953251128675613, -0.70710678118654752440, -0.38268343236508977173};
-    const R c = (R)cs[m], s = (R)(INV ? sn[m] : -sn[m]);
-    return mk<R>(a.x * c - a.y * s, a.x * s + a.y * c);
+    if constexpr (fixed::is_fixed<R>::value) {
+        return fixed::w16<INV, m>(a);
+    } else {
+        if (m == 0) return a;
+        if (m == 4) return rot<R, INV>(a);
+        if (m == 8) return mk<R>(-a.x, -a.y);
+        if (m == 12) return rot<R, !INV>(a);
+        // cos and sin of 2 pi m / 16
+        constexpr double cs[16] = {1.0, 0.92387953251128675613, 0.70710678118654752440, 0.38268343236508977173,
+                                   0.0, -0.38268343236508977173, -0.70710678118654752440, -0.92387953251128675613,
+                                   -1.0, -0.92387953251128675613, -0.70710678118654752440, -0.38268343236508977173,
+                                   0.0, 0.38268343236508977173, 0.70710678118654752440, 0.92387953251128675613};
+        constexpr double sn[16] = {0.0, 0.38268343236508977173, 0.70710678118654752440, 0.92387953251128675613,
+                                   1.0, 0.92387953251128675613, 0.70710678118654752440, 0.38268343236508977173,
+                                   0.0, -0.38268343236508977173, -0.70710678118654752440, -0.92387953251128675613,
+                                   -1.0, -0.92387953251128675613, -0.70710678118654752440, -0.38268343236508977173};
+        const R c = (R)cs[m], s = (R)(INV ? sn[m] : -sn[m]);
+        return mk<R>(a.x * c - a.y * s, a.x * s + a.y * c);
+    }
 }
 
 // 16-point DFT in registers (q = q1 + 4 q2, k = k2 + 4 k1); v[k] holds y_k on return
-template <typename R, bool INV, bool PK> __device__ __forceinline__ void dft16(C<R> v[16]) {
+template <typename R, bool INV, bool PK> __host__ __device__ __forceinline__ void dft16(C<R> v[16]) {
 #pragma unroll
     for (int q1 = 0; q1 < 4; ++q1) dft4<R, INV, PK>(v[q1], v[q1 + 4], v[q1 + 8], v[q1 + 12]);
     // v[q1 + 4 k2] = b(q1, k2); twiddle by w16^(q1 k2)
@@ -120,7 +137,7 @@ template <typename R, bool INV, bool PK> __device__ __forceinline__ void dft16(C
 }
 
 // 8-point DFT (q = q1 + 2 q2, k = k2 + 4 k1)
-template <typename R, bool INV, bool PK> __device__ __forceinline__ void dft8(C<R> v[8]) {
+template <typename R, bool INV, bool PK> __host__ __device__ __forceinline__ void dft8(C<R> v[8]) {
     dft4<R, INV, PK>(v[0], v[2], v[4], v[6]);
     dft4<R, INV, PK>(v[1], v[3], v[5], v[7]);
     // v[q1 + 2 k2] = b(q1, k2); twiddle q1 = 1 by w8^k2 = w16^(2 k2)
@@ -139,7 +156,7 @@ template <typename R, bool INV, bool PK> __device__ __forceinline__ void dft8(C<
     for (int k = 0; k < 8; ++k) v[k] = t[k];
 }
 
-template <typename R, bool INV, int RADIX, bool PK> __device__ __forceinline__ void dft_small(C<R> *v) {
+template <typename R, bool INV, int RADIX, bool PK> __host__ __device__ __forceinline__ void dft_small(C<R> *v) {
     if (RADIX == 2) dft2<R, INV, PK>(v[0], v[1]);
     if (RADIX == 4) dft4<R, INV, PK>(v[0], v[1], v[2], v[3]);
     if (RADIX == 8) dft8<R, INV, PK>(v);
@@ -184,8 +201,14 @@ __device__ __forceinline__ void st_cluster(uint32_t a, float2 v) {
 __device__ __forceinline__ void st_cluster(uint32_t a, double2 v) {
     asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
 }
+__device__ __forceinline__ void st_cluster(uint32_t a, longlong2 v) {
+    asm volatile("st.shared::cluster.v2.b64 [%0], {%1, %2};" ::"r"(a), "l"(v.x), "l"(v.y) : "memory");
+}
 __device__ __forceinline__ void ld_cluster(uint32_t a, float2 &v) {
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void ld_cluster(uint32_t a, longlong2 &v) {
+    asm volatile("ld.shared::cluster.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a) : "memory");
 }
 __device__ __forceinline__ void ld_cluster(uint32_t a, double2 &v) {
     asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
@@ -233,24 +256,34 @@ template <typename R, int LOG2N, bool PK = false, int CS = 1> struct LineFFT {
     // their line count instead: col_line_stride in lbm_internal.cuh)
     static constexpr int STRIDE = SMEM + 2;
     typedef C<R> CT;
+    static constexpr bool FIXED = fixed::is_fixed<R>::value;
+    static constexpr int TWIDDLED = LOG2N >= 5 ? (LOG2N - 1) / 4 : 0;  // radix-16 passes with outer twiddles
 
-    static __device__ __forceinline__ int pad(int p) { return p + (p >> 4); }
+    static __host__ __device__ __forceinline__ int pad(int p) { return p + (p >> 4); }
     // padded index of this CTA's first position (0 without a cluster split)
     static __device__ __forceinline__ int pad_base() {
         if constexpr (CS == 1) return 0;
         else return pad((int)cluster_rank() * NL);
     }
     // position of point e of thread t in the input layout of radix-16 pass P
-    template <int P> static __device__ __forceinline__ int pos16(int t, int e) {
+    template <int P> static __host__ __device__ __forceinline__ int pos16(int t, int e) {
         constexpr int S = N >> (4 * P), M = S >> 4;
         return (t / M) * S + (t & (M - 1)) + M * e;
     }
 
-    template <int P, bool INV> static __device__ __forceinline__ void pass16(CT v[16], int t, const CT *__restrict__ tw) {
+    template <int P, bool INV> static __host__ __device__ __forceinline__ void pass16(CT v[16], int t, const CT *__restrict__ tw) {
         constexpr int S = N >> (4 * P), M = S >> 4;
         const int j = t & (M - 1);
         const CT *twp = tw + twiddle_offset(N, P) + j;  // root of (j, k) at twp[(k - 1) M]
-        if (INV) {
+        if constexpr (FIXED) {  // a twiddled pass also scales every point by 1/4 (root 1 as well)
+            if (!INV) dft16<R, false, PK>(v);
+            if (M > 1) {
+                v[0] = fixed::quarter(v[0]);
+#pragma unroll
+                for (int k = 1; k < 16; ++k) v[k] = INV ? mulc<R>(v[k], twp[(k - 1) * M]) : mul<R>(v[k], twp[(k - 1) * M]);
+            }
+            if (INV) dft16<R, true, PK>(v);
+        } else if (INV) {
             if (M > 1 && j) {
 #pragma unroll
                 for (int k = 1; k < 16; ++k) v[k] = mulc<R>(v[k], twp[(k - 1) * M]);
@@ -265,19 +298,19 @@ template <typename R, int LOG2N, bool PK = false, int CS = 1> struct LineFFT {
         }
     }
 
-    template <int P> static __device__ __forceinline__ void store16(const CT v[E], CT *buf, int t, int pb = 0) {
+    template <int P> static __host__ __device__ __forceinline__ void store16(const CT v[E], CT *buf, int t, int pb = 0) {
 #pragma unroll
         for (int e = 0; e < E; ++e) buf[pad(pos16<P>(t, e)) - pb] = v[e];
     }
-    template <int P> static __device__ __forceinline__ void load16(CT v[E], const CT *buf, int t, int pb = 0) {
+    template <int P> static __host__ __device__ __forceinline__ void load16(CT v[E], const CT *buf, int t, int pb = 0) {
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = buf[pad(pos16<P>(t, e)) - pb];
     }
-    static __device__ __forceinline__ void storeF(const CT v[E], CT *buf, int t, int pb = 0) {
+    static __host__ __device__ __forceinline__ void storeF(const CT v[E], CT *buf, int t, int pb = 0) {
 #pragma unroll
         for (int e = 0; e < E; ++e) buf[pad(t * E + e) - pb] = v[e];
     }
-    static __device__ __forceinline__ void loadF(CT v[E], const CT *buf, int t, int pb = 0) {
+    static __host__ __device__ __forceinline__ void loadF(CT v[E], const CT *buf, int t, int pb = 0) {
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = buf[pad(t * E + e) - pb];
     }

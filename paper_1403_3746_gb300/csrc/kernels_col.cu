@@ -54,7 +54,7 @@ template <typename R> static int jobs_acc(const ColArgs<R> &a, int njobs) {
 
 template <typename R, int LOG2N, int CS, bool ACC>
 static cudaError_t launch_col_cs_t(const ColArgs<R> &a, int njobs, size_t smem, cudaStream_t s) {
-    using F = reg::LineFFT<R, LOG2N, true, CS>;
+    using F = reg::Line<R, LOG2N, true, CS>;
     dim3 grid((a.nx / a.W) * CS, njobs, a.nb > 0 ? a.nb : 1);
     if constexpr (CS == 1) {
         cudaError_t e = allow_smem(col_deriv_kernel<R, LOG2N, ACC>);
@@ -83,7 +83,7 @@ static cudaError_t launch_col_cs_t(const ColArgs<R> &a, int njobs, size_t smem, 
 
 template <typename R, int LOG2N, int CS> static cudaError_t launch_col_cs(const ColArgs<R> &a, int njobs, size_t smem,
                                                                            cudaStream_t s) {
-    using F = reg::LineFFT<R, LOG2N, true, CS>;
+    using F = reg::Line<R, LOG2N, true, CS>;
     if (smem < (size_t)(a.W / 2) * col_line_stride(LOG2N, sizeof(R), CS) * sizeof(typename F::CT))
         return cudaErrorInvalidValue;
     const int acc = jobs_acc(a, njobs);
@@ -119,7 +119,7 @@ template <typename R, int LOG2N> static cudaError_t launch_col_n(const ColArgs<R
 template <typename R, int LOG2N, bool ACC>
 __global__ void __launch_bounds__(PassThreads<R>::value, PassThreads<R>::min_blocks)
     col_tma_kernel(const __grid_constant__ ColTmaArgs<R> a) {
-    using F = reg::LineFFT<R, LOG2N, true>;
+    using F = reg::Line<R, LOG2N, true>;
     using CT = typename F::CT;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const ColArgs<R> &c = a.c;
@@ -175,9 +175,9 @@ __global__ void __launch_bounds__(PassThreads<R>::value, PassThreads<R>::min_blo
 #pragma unroll
         for (int e = 0; e < F::E; ++e) v[e] = st[(size_t)(t + F::G * e) * L + l];  // row t + G e, columns 2l, 2l+1
         CT *buf = st + l * col_line_stride(LOG2N, sizeof(R), 1);
-        F::template forward<reg::SyncCta>(v, buf, t, c.ay.tw);
-        F::multiply(v, t, jb.order, jb.c, c.ay.k1, c.ay.k2);
-        F::template inverse<reg::SyncCta>(v, buf, t, c.ay.tw);
+        typename F::Scale sc = F::template forward<reg::SyncCta>(v, buf, t, c.ay, L);
+        F::multiply(v, t, jb.order, jb.c, c.ay, sc);
+        F::template inverse<reg::SyncCta>(v, buf, t, c.ay, sc, L);
         const size_t rso = (size_t)(jb.ld_out >> 1), rsi = (size_t)(jb.ld_in >> 1);
         CT *out = reinterpret_cast<CT *>(jb.out + (size_t)z_of(it) * c.ny * jb.ld_out + tile_of(it) * W + 2 * l);
         const CT *inp = reinterpret_cast<const CT *>(jb.in + (size_t)z_of(it) * c.ny * jb.ld_in + tile_of(it) * W + 2 * l);
@@ -229,7 +229,7 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 
 template <typename R, int LOG2N, bool ACC>
 static cudaError_t launch_col_tma_t(const ColTmaArgs<R> &a, size_t smem, cudaStream_t s) {
-    using F = reg::LineFFT<R, LOG2N>;
+    using F = reg::Line<R, LOG2N, true>;
     const int threads = (a.c.W / 2) * F::G;
     if (threads > PassThreads<R>::value ||
         a.stage_bytes < (unsigned)((a.c.W / 2) * col_line_stride(LOG2N, sizeof(R), 1) * sizeof(typename F::CT)))

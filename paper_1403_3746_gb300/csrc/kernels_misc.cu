@@ -191,7 +191,7 @@ __global__ void field_out_kernel(const R *src, int ld, double *out, int nx, int 
 // transformed in place (out = in): every thread reads its points before any is written back.
 template <typename R, int LOG2N>
 __global__ void __launch_bounds__(MaxThreads<R>::value) row_deriv_kernel(const __grid_constant__ RowDerivArgs<R> a) {
-    using F = reg::LineFFT<R, LOG2N>;
+    using F = reg::Line<R, LOG2N, false>;
     using CT = typename F::CT;
     constexpr int G = F::G, E = F::E;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -208,9 +208,9 @@ __global__ void __launch_bounds__(MaxThreads<R>::value) row_deriv_kernel(const _
         v[e] = reg::mk<R>(a.in[ka][g], kb < a.nin ? a.in[kb][g] : R(0));
     }
     CT *buf = sb + (size_t)slot * F::STRIDE;
-    F::template forward<reg::SyncCta>(v, buf, t, a.ax.tw);
-    F::multiply(v, t, a.order == 2 ? 2 : 1, R(1), a.ax.k1, a.ax.k2);
-    F::template inverse<reg::SyncCta>(v, buf, t, a.ax.tw);
+    typename F::Scale sc = F::template forward<reg::SyncCta>(v, buf, t, a.ax, 1);
+    F::multiply(v, t, a.order == 2 ? 2 : 1, R(1), a.ax, sc);
+    F::template inverse<reg::SyncCta>(v, buf, t, a.ax, sc, 1);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const size_t g = row + t + G * e;
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(MaxThreads<R>::value) row_deriv_kernel(const _
 
 template <typename R, int LOG2N> static cudaError_t launch_row_deriv_n(const RowDerivArgs<R> &a, size_t smem,
                                                                        cudaStream_t s) {
-    using F = reg::LineFFT<R, LOG2N>;
+    using F = reg::Line<R, LOG2N, false>;
     if (smem < (size_t)((a.nin + 1) / 2) * a.rows * F::STRIDE * sizeof(typename F::CT)) return cudaErrorInvalidValue;
     cudaError_t e = allow_smem(row_deriv_kernel<R, LOG2N>);
     if (e != cudaSuccess) return e;

@@ -32,7 +32,7 @@ __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(PassThreads<R>::val
 
 template <typename R, int LOG2N, int CS> static cudaError_t launch_update_cs(const UpdateArgs<R> &a, size_t smem,
                                                                               cudaStream_t s) {
-    using F = reg::LineFFT<R, LOG2N, true, CS>;
+    using F = reg::Line<R, LOG2N, true, CS>;
     constexpr bool MS = sizeof(R) == 4;  // float32: moment-space collision
     cudaError_t e;
     if constexpr (CS == 1) e = allow_smem(update_row_kernel<R, LOG2N, MS>);
@@ -74,7 +74,7 @@ template <typename R, int LOG2N> static cudaError_t launch_update_n(const Update
 
 template <typename R, int LOG2N> static cudaError_t launch_macro_n(const MacroArgs<R> &a, size_t smem,
                                                                    cudaStream_t s) {
-    using F = reg::LineFFT<R, LOG2N>;
+    using F = reg::Line<R, LOG2N, true>;
     // three line buffers per row; refuse less
     const size_t need = (size_t)3 * a.rows * F::STRIDE * sizeof(typename F::CT);
     if (smem < need) return cudaErrorInvalidValue;

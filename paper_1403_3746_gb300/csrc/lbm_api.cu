@@ -132,9 +132,12 @@ struct lbm_ctx {
     // per-axis tables
     double2 *tw64x = nullptr, *tw64y = nullptr;
     float2 *tw32x = nullptr, *tw32y = nullptr;
-    double *k1x = nullptr, *k2x = nullptr, *k1y = nullptr, *k2y = nullptr;
+    // float64 lines in fixed point (fft_fixed.cuh): roots, multipliers and their exponents
+    longlong2 *twfx = nullptr, *twfy = nullptr;
+    long long *k1x = nullptr, *k2x = nullptr, *k1y = nullptr, *k2y = nullptr;
+    int p1x = 0, p2x = 0, p1y = 0, p2y = 0, pfx = 0, pfy = 0;
     float *k1x32 = nullptr, *k2x32 = nullptr, *k1y32 = nullptr, *k2y32 = nullptr;
-    double *kfx = nullptr, *kfy = nullptr;  // solution filter W(m) / N per axis (params filter_alpha > 0)
+    long long *kfx = nullptr, *kfy = nullptr;  // solution filter W(m) / N per axis (params filter_alpha > 0)
     float *kfx32 = nullptr, *kfy32 = nullptr;
     double minv[256];
 
@@ -210,7 +213,8 @@ struct LaunchTimer {
 
 template <typename R> Axis<R> axis(const lbm_ctx *c, bool xdir);
 template <> Axis<double> axis<double>(const lbm_ctx *c, bool xdir) {
-    return xdir ? Axis<double>{c->tw64x, c->k1x, c->k2x, c->lx} : Axis<double>{c->tw64y, c->k1y, c->k2y, c->ly};
+    return xdir ? Axis<double>{c->twfx, c->k1x, c->k2x, c->lx, c->p1x, c->p2x}
+                : Axis<double>{c->twfy, c->k1y, c->k2y, c->ly, c->p1y, c->p2y};
 }
 template <> Axis<float> axis<float>(const lbm_ctx *c, bool xdir) {
     return xdir ? Axis<float>{c->tw32x, c->k1x32, c->k2x32, c->lx}
@@ -446,7 +450,8 @@ int run_stage(lbm_ctx *c, int stage, int passes = PASS_ALL) {
 // field, then the moments of the filtered f for the next step.
 template <typename R> Axis<R> filter_axis(const lbm_ctx *c, bool xdir);
 template <> Axis<double> filter_axis<double>(const lbm_ctx *c, bool xdir) {
-    return xdir ? Axis<double>{c->tw64x, c->k1x, c->kfx, c->lx} : Axis<double>{c->tw64y, c->k1y, c->kfy, c->ly};
+    return xdir ? Axis<double>{c->twfx, c->k1x, c->kfx, c->lx, c->p1x, c->pfx}
+                : Axis<double>{c->twfy, c->k1y, c->kfy, c->ly, c->p1y, c->pfy};
 }
 template <> Axis<float> filter_axis<float>(const lbm_ctx *c, bool xdir) {
     return xdir ? Axis<float>{c->tw32x, c->k1x32, c->kfx32, c->lx} : Axis<float>{c->tw32y, c->k1y32, c->kfy32, c->ly};
@@ -865,6 +870,8 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
     parts.push_back({reinterpret_cast<void **>(&c->tw64y), (size_t)ny * 16});
     parts.push_back({reinterpret_cast<void **>(&c->tw32x), (size_t)nx * 8});
     parts.push_back({reinterpret_cast<void **>(&c->tw32y), (size_t)ny * 8});
+    parts.push_back({reinterpret_cast<void **>(&c->twfx), (size_t)nx * sizeof(longlong2)});
+    parts.push_back({reinterpret_cast<void **>(&c->twfy), (size_t)ny * sizeof(longlong2)});
     parts.push_back({reinterpret_cast<void **>(&c->k1x), (size_t)nx * 8});
     parts.push_back({reinterpret_cast<void **>(&c->k2x), (size_t)nx * 8});
     parts.push_back({reinterpret_cast<void **>(&c->k1y), (size_t)ny * 8});
@@ -904,10 +911,16 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
             k1f[pos] = (float)k1[pos];
             k2f[pos] = (float)k2[pos];
         }
-        double *dk1 = ax == 0 ? c->k1x : c->k1y, *dk2 = ax == 0 ? c->k2x : c->k2y;
+        long long *dk1 = ax == 0 ? c->k1x : c->k1y, *dk2 = ax == 0 ? c->k2x : c->k2y;
+        std::vector<long long> k1i(N), k2i(N), kfi(N);
+        std::vector<longlong2> twf(N);
+        fixed_twiddles(N, twf.data());
+        (ax == 0 ? c->p1x : c->p1y) = fixed_multipliers(N, k1.data(), k1i.data());
+        (ax == 0 ? c->p2x : c->p2y) = fixed_multipliers(N, k2.data(), k2i.data());
         float *fk1 = ax == 0 ? c->k1x32 : c->k1y32, *fk2 = ax == 0 ? c->k2x32 : c->k2y32;
-        e = cudaMemcpy(dk1, k1.data(), N * 8, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(dk2, k2.data(), N * 8, cudaMemcpyHostToDevice);
+        e = cudaMemcpy(ax == 0 ? c->twfx : c->twfy, twf.data(), N * sizeof(longlong2), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(dk1, k1i.data(), N * 8, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(dk2, k2i.data(), N * 8, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(fk1, k1f.data(), N * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(fk2, k2f.data(), N * 4, cudaMemcpyHostToDevice);
         // the solution filter's table (unused while filter_alpha = 0)
@@ -915,7 +928,8 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
         std::vector<float> kff(N);
         filter_table(N, params->filter_alpha, params->filter_p, kf.data());
         for (int pos = 0; pos < N; ++pos) kff[pos] = (float)kf[pos];
-        if (e == cudaSuccess) e = cudaMemcpy(ax == 0 ? c->kfx : c->kfy, kf.data(), N * 8, cudaMemcpyHostToDevice);
+        (ax == 0 ? c->pfx : c->pfy) = fixed_multipliers(N, kf.data(), kfi.data());
+        if (e == cudaSuccess) e = cudaMemcpy(ax == 0 ? c->kfx : c->kfy, kfi.data(), N * 8, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(ax == 0 ? c->kfx32 : c->kfy32, kff.data(), N * 4, cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -2303,6 +2317,40 @@ void derivative_tables(int N, double d, double win_alpha, double win_p, double *
         k1[at] = ke / N;
         k2[at] = -ke * ke / N;
     }
+}
+
+void fixed_twiddles(int N, longlong2 *out) {
+    // exp(-2 pi i a / 4096), a < 4096, from one octant in long double (at least 64 bits), once
+    static const std::vector<longlong2> roots = [] {
+        const int M = 4096, O = M / 8;
+        std::vector<long long> c(O + 1), s(O + 1);
+        const long double w = acosl(-1.0L) * 2 / M;
+        for (int a = 0; a <= O; ++a) {
+            c[a] = llrintl(cosl(w * a) * 0x1p62L);
+            s[a] = llrintl(sinl(w * a) * 0x1p62L);
+        }
+        std::vector<longlong2> r(M);
+        for (int a = 0; a < M; ++a) {
+            const int q = a / (2 * O), b = a % (2 * O);  // quadrant and angle within it
+            const long long x = b <= O ? c[b] : s[2 * O - b], y = b <= O ? s[b] : c[2 * O - b];
+            const long long re = q == 0 ? x : q == 1 ? -y : q == 2 ? -x : y, im = q == 0 ? y : q == 1 ? x : q == 2 ? -y : -x;
+            r[a] = longlong2{fixed::balance(re), fixed::balance(-im)};
+        }
+        return r;
+    }();
+    for (int i = 0; i < N; ++i) {
+        const int a = reg::twiddle_exponent(N, i);
+        out[i] = roots[a > 0 ? a * (4096 / N) : 0];
+    }
+}
+
+int fixed_multipliers(int N, const double *k, long long *out) {
+    double top = 0.0;
+    for (int i = 0; i < N; ++i) top = std::max(top, std::fabs(k[i]));
+    int p = 0;
+    if (top > 0) std::frexp(top, &p);  // |k| 2^-p < 1
+    for (int i = 0; i < N; ++i) out[i] = fixed::balance(std::llrint(std::ldexp(k[i], 62 - p)));
+    return p;
 }
 
 void filter_table(int N, double alpha, double p, double *kf) {

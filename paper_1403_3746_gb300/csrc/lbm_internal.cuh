@@ -16,7 +16,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "fft_reg.cuh"
+#include "fft_line.cuh"
 #include "lbm_d2v16.h"
 #include "tma.cuh"
 
@@ -141,6 +141,11 @@ void derivative_tables(int N, double d, double win_alpha, double win_p, double *
 // of the correction times the spectrum, so the rounding of the transforms touches only the small
 // removed part and the mean (W(0) = 1) is kept exactly (lbm_api.cu).
 void filter_table(int N, double alpha, double p, double *kf);
+// The float64 path's tables in fixed point (fft_fixed.cuh): the roots of a line of N points in
+// the layout of fft_reg.cuh, scaled to 2^62, and a multiplier table k = out 2^(p - 62), |out| <= 2^62,
+// both in balanced halves; the second returns p (lbm_api.cu).
+void fixed_twiddles(int N, longlong2 *out);
+int fixed_multipliers(int N, const double *k, long long *out);
 
 // Launch geometry of the four passes for an nx x ny grid and an element size (lbm_api.cu):
 // column tile width and shared memory, rows per CTA and shared memory of the row kernels.
@@ -161,14 +166,6 @@ struct Geometry {
     int flux_kind = 0;          // flux column pass: the same choice (width fluxW)
 };
 void pass_geometry(int nx, int ny, size_t esize, Geometry *g);
-
-// twiddles and derivative multipliers of one axis (digit-reversed order, see fft_reg.cuh)
-template <typename R> struct Axis {
-    const typename cplx<R>::T *tw;  // exp(-2 pi i k/N), k < N
-    const R *k1;                    // k_eff(m(p)) / N, 0 at Nyquist
-    const R *k2;                    // -k_eff(m(p))^2 / N, 0 at Nyquist
-    int log2n;
-};
 
 // ---- HBM layout ------------------------------------------------------------------------
 // Row-interleaved field blocks: a group of NF fields over an nx x ny grid is stored as

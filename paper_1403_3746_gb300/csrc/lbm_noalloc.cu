@@ -29,10 +29,9 @@ constexpr int kMaxBlocks = 1024;            // reduction blocks
 constexpr size_t kOffRx = 0;                             // d_x rho   [kMaxNodes]
 constexpr size_t kOffRy = kOffRx + kMaxNodes;            // d_y rho   [kMaxNodes]
 constexpr size_t kOffPart = kOffRy + kMaxNodes;          // partials  [kMaxBlocks * 5]
-constexpr size_t kOffK = kOffPart + kMaxBlocks * 5;      // k1x, k2x, k1y, k2y [4 * kMaxN]
-constexpr size_t kOffTw64 = kOffK + 4 * kMaxN;           // double2 twiddles x, y [2 * kMaxN * 2]
-constexpr size_t kOffTw32 = kOffTw64 + 4 * kMaxN;        // float2 twiddles x, y [2 * kMaxN]
-constexpr size_t kScratchDoubles = kOffTw32 + 2 * kMaxN;  // about 16.3 MiB in total
+constexpr size_t kOffK = kOffPart + kMaxBlocks * 5;      // multipliers k1 of x, y [2 * kMaxN]
+constexpr size_t kOffTw = kOffK + 2 * kMaxN;             // longlong2 roots of x, y [2 * kMaxN * 2]
+constexpr size_t kScratchDoubles = kOffTw + 4 * kMaxN;   // about 16.2 MiB in total
 
 static __device__ __align__(256) double g_noalloc_scratch[kScratchDoubles];
 
@@ -98,16 +97,20 @@ extern "C" int lbm_diagnostics_noalloc(int nx, int ny, double dx, double dy, dou
     int rc = scratch_address(&sc);
     if (rc) return rc;
 
-    // derivative tables of both axes, rebuilt by every call
-    double *k1x = sc + kOffK, *k2x = k1x + kMaxN, *k1y = k2x + kMaxN, *k2y = k1y + kMaxN;
-    double2 *twx = reinterpret_cast<double2 *>(sc + kOffTw64), *twy = twx + kMaxN;
-    float2 *twx32 = reinterpret_cast<float2 *>(sc + kOffTw32), *twy32 = twx32 + kMaxN;
-    NA_TRY(launch_twiddles(twx, twx32, nx, s));
-    NA_TRY(launch_twiddles(twy, twy32, ny, s));
-    std::vector<double> tab(4 * (size_t)kMaxN);
-    derivative_tables(nx, dx, win_alpha, win_p, tab.data(), tab.data() + kMaxN, keff_terms);
-    derivative_tables(ny, dy, win_alpha, win_p, tab.data() + 2 * kMaxN, tab.data() + 3 * kMaxN, keff_terms);
-    NA_TRY(cudaMemcpyAsync(k1x, tab.data(), 4 * (size_t)kMaxN * sizeof(double), cudaMemcpyHostToDevice, s));
+    // derivative tables of both axes (first derivatives, in fixed point), rebuilt by every call
+    long long *k1x = reinterpret_cast<long long *>(sc + kOffK), *k1y = k1x + kMaxN;
+    longlong2 *twx = reinterpret_cast<longlong2 *>(sc + kOffTw), *twy = twx + kMaxN;
+    std::vector<double> k1(kMaxN), k2(kMaxN);
+    std::vector<long long> ktab(2 * (size_t)kMaxN);
+    std::vector<longlong2> twtab(2 * (size_t)kMaxN);
+    derivative_tables(nx, dx, win_alpha, win_p, k1.data(), k2.data(), keff_terms);
+    const int p1x = fixed_multipliers(nx, k1.data(), ktab.data());
+    derivative_tables(ny, dy, win_alpha, win_p, k1.data(), k2.data(), keff_terms);
+    const int p1y = fixed_multipliers(ny, k1.data(), ktab.data() + kMaxN);
+    fixed_twiddles(nx, twtab.data());
+    fixed_twiddles(ny, twtab.data() + kMaxN);
+    NA_TRY(cudaMemcpyAsync(k1x, ktab.data(), ktab.size() * sizeof(long long), cudaMemcpyHostToDevice, s));
+    NA_TRY(cudaMemcpyAsync(twx, twtab.data(), twtab.size() * sizeof(longlong2), cudaMemcpyHostToDevice, s));
 
     // d_y rho (column pass) and d_x rho (row pass) into the scratch fields
     Geometry geo;
@@ -118,7 +121,7 @@ extern "C" int lbm_diagnostics_noalloc(int nx, int ny, double dx, double dy, dou
     ca.ny = ny;
     ca.W = W;
     ca.log2W = log2i(W);
-    ca.ay = Axis<double>{twy, k1y, k2y, log2i(ny)};
+    ca.ay = Axis<double>{twy, k1y, nullptr, log2i(ny), p1y, 0};
     ca.jobs[0] = ColJob<double>{rho, sc + kOffRy, nx, nx, 1, 1.0};
     NA_TRY(launch_col<double>(ca, 1, geo.col_smem, s));
     RowDerivArgs<double> ra{};
@@ -130,7 +133,7 @@ extern "C" int lbm_diagnostics_noalloc(int nx, int ny, double dx, double dy, dou
     ra.ny = ny;
     ra.rows = geo.rows_rowd;
     ra.order = 1;
-    ra.ax = Axis<double>{twx, k1x, k2x, log2i(nx)};
+    ra.ax = Axis<double>{twx, k1x, nullptr, log2i(nx), p1x, 0};
     NA_TRY(launch_row_deriv<double>(ra, geo.rowd_smem, s));
 
     // per-block partial sums, then the final reduction on the host

@@ -16,21 +16,18 @@ namespace lbm {
 // filter's correction), a separate instantiation so that the plain passes keep their registers.
 template <typename R, int LOG2N, int CS, bool EXTRA = false, bool ACC = false>
 __device__ __forceinline__ void col_tile(const ColArgs<R> &a, int jobi, int z, int tile, unsigned rank) {
-    using F = reg::LineFFT<R, LOG2N, true, CS>;
+    using F = reg::Line<R, LOG2N, true, CS>;
     using CT = typename F::CT;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     CT *sbuf = reinterpret_cast<CT *>(smem_raw);
     const ColJob<R> &job = a.jobs[jobi];
     const int L = a.W >> 1;
-    if (EXTRA && (int)threadIdx.x >= L * F::GL) {
-        if constexpr (CS == 1) {
-            F::template idle<reg::SyncCta>();
-            F::template idle<reg::SyncCta>();
-        } else {
+    if constexpr (EXTRA) {
+        if ((int)threadIdx.x >= L * F::GL) {
             F::template idle_forward<reg::SyncCta>();
             F::template idle_inverse<reg::SyncCta>();
+            return;
         }
-        return;
     }
     const int l = threadIdx.x & (L - 1);
     const int t = (int)rank * F::GL + (threadIdx.x >> (a.log2W - 1));  // thread of the line, across the cluster
@@ -43,9 +40,9 @@ __device__ __forceinline__ void col_tile(const ColArgs<R> &a, int jobi, int z, i
 #pragma unroll
     for (int e = 0; e < F::E; ++e) v[e] = __ldcg(in + (size_t)(t + F::G * e) * rsi);  // L2 only: single use
     CT *buf = sbuf + l * col_line_stride(LOG2N, sizeof(R), CS);
-    F::template forward<reg::SyncCta>(v, buf, t, a.ay.tw);
-    F::multiply(v, t, job.order, job.c, a.ay.k1, a.ay.k2);
-    F::template inverse<reg::SyncCta>(v, buf, t, a.ay.tw);
+    typename F::Scale sc = F::template forward<reg::SyncCta>(v, buf, t, a.ay, L);
+    F::multiply(v, t, job.order, job.c, a.ay, sc);
+    F::template inverse<reg::SyncCta>(v, buf, t, a.ay, sc, L);
     if constexpr (ACC) {  // out = in + result; each position is read and written by this thread only
 #pragma unroll
         for (int e = 0; e < F::E; ++e) {
@@ -108,7 +105,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
 // its five partial values to a.diag_partial, as the diagnostics kernel would.
 template <typename R, int LOG2N, bool SERIAL, bool EXTRA = false, bool RHO64 = false, bool DIAG = false>
 __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
-    using F = reg::LineFFT<R, LOG2N, true>;
+    using F = reg::Line<R, LOG2N, true>;
     using CT = typename F::CT;
     constexpr int NX = F::N, G = F::G, E = F::E, SM = F::STRIDE;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -136,10 +133,10 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
     for (int kind = my_kind; kind <= (SERIAL ? 1 : my_kind); ++kind) {
         if (!active) {  // the barriers of the line groups (A then B in turn when SERIAL, else B)
             for (int k = 0; k < (SERIAL ? 2 : 1); ++k) {
-                F::template idle<reg::SyncCta>();
-                F::template idle<reg::SyncCta>();
+                F::template idle_forward<reg::SyncCta>();
+                F::template idle_inverse<reg::SyncCta>();
                 reg::cta_barrier();
-                if (!SERIAL || k == 0) F::template idle<reg::SyncCta>();
+                if (!SERIAL || k == 0) F::template idle_inverse<reg::SyncCta>();
                 reg::cta_barrier();
             }
             break;
@@ -151,19 +148,21 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
             v[e] = kind == 0 ? reg::mk<R>(__ldcg(mrow + M_RHO * NX + x), __ldcg(mrow + M_T * NX + x))
                              : reg::mk<R>(__ldcg(mrow + M_UX * NX + x), __ldcg(mrow + M_UY * NX + x));
         }
-        F::template forward<reg::SyncCta>(v, O1, t, a.ax.tw);
+        const typename F::Scale sc0 = F::template forward<reg::SyncCta>(v, O1, t, a.ax, 1);
         if (kind == 0) F::storeF(v, O2, t);  // keep the spectrum of A for d_xx rho (thread-private slots)
-        F::multiply(v, t, 1, R(1), a.ax.k1, a.ax.k2);
-        F::template inverse<reg::SyncCta>(v, O1, t, a.ax.tw);
+        typename F::Scale sc = sc0;
+        F::multiply(v, t, 1, R(1), a.ax, sc);
+        F::template inverse<reg::SyncCta>(v, O1, t, a.ax, sc, 1);
         reg::cta_barrier();
 #pragma unroll
         for (int e = 0; e < E; ++e) O1[t + G * e] = v[e];
         if (kind == 0) {
             F::loadF(v, O2, t);
-            F::multiply(v, t, 2, R(1), a.ax.k1, a.ax.k2);
-            F::template inverse<reg::SyncCta>(v, O2, t, a.ax.tw);
+            sc = sc0;
+            F::multiply(v, t, 2, R(1), a.ax, sc);
+            F::template inverse<reg::SyncCta>(v, O2, t, a.ax, sc, 1);
         } else if (!SERIAL) {
-            F::template idle<reg::SyncCta>();
+            F::template idle_inverse<reg::SyncCta>();
         }
         reg::cta_barrier();
         if (kind == 0) {
@@ -250,15 +249,18 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
     // round 2: d_x of (Q_x, S_xx) on line A and of (S_xy, div u) on line B
     for (int kind = my_kind; kind <= (SERIAL ? 1 : my_kind); ++kind) {
         if (!active) {
-            for (int k = 0; k < (SERIAL ? 4 : 2); ++k) F::template idle<reg::SyncCta>();
+            for (int k = 0; k < (SERIAL ? 2 : 1); ++k) {
+                F::template idle_forward<reg::SyncCta>();
+                F::template idle_inverse<reg::SyncCta>();
+            }
             break;
         }
         CT *O1 = buf1(kind);
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e] = O1[t + G * e];
-        F::template forward<reg::SyncCta>(v, O1, t, a.ax.tw);
-        F::multiply(v, t, 1, R(1), a.ax.k1, a.ax.k2);
-        F::template inverse<reg::SyncCta>(v, O1, t, a.ax.tw);
+        typename F::Scale sc = F::template forward<reg::SyncCta>(v, O1, t, a.ax, 1);
+        F::multiply(v, t, 1, R(1), a.ax, sc);
+        F::template inverse<reg::SyncCta>(v, O1, t, a.ax, sc, 1);
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int x = t + G * e;
@@ -611,7 +613,7 @@ __device__ __forceinline__ void update_node(const UpdateArgs<R> &a, const Update
 // transforms leave in its own shared memory.
 template <typename R, int LOG2N, bool MOMENT_SPACE, int CS>
 __device__ __forceinline__ void update_rows(const UpdateArgs<R> &a, const UpdateConst<R> &kc, int blk, unsigned rank) {
-    using F = reg::LineFFT<R, LOG2N, true, CS>;
+    using F = reg::Line<R, LOG2N, true, CS>;
     using CT = typename F::CT;
     constexpr int NX = F::N, G = F::G, E = F::E, SM = F::STRIDE, NL = F::NL;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -663,9 +665,9 @@ __device__ __forceinline__ void update_rows(const UpdateArgs<R> &a, const Update
                 CT v[E];
 #pragma unroll
                 for (int e = 0; e < E; ++e) v[e] = reg::mk<R>(ldcg(fa + t + G * e), ldcg(fb + t + G * e));
-                F::template forward<reg::SyncCta>(v, buf, t, a.ax.tw);
-                F::multiply(v, t, 1, a.cx[p], a.ax.k1, a.ax.k2);  // -h v_x folded in
-                F::template inverse<reg::SyncCta>(v, buf, t, a.ax.tw);
+                typename F::Scale sc = F::template forward<reg::SyncCta>(v, buf, t, a.ax, 1);
+                F::multiply(v, t, 1, a.cx[p], a.ax, sc);  // -h v_x folded in
+                F::template inverse<reg::SyncCta>(v, buf, t, a.ax, sc, 1);
                 if constexpr (CS == 1) reg::cta_barrier();  // (a split inverse ends with a cluster barrier)
                 F::store_natural(v, buf, t);
             } else {
