@@ -53,7 +53,7 @@ template <typename R>
 __device__ __forceinline__ void batch_update(const UpdateArgs<R> &u, const UpdateConst<R> &kc, int blk) {
     switch (u.ax.log2n) {
 #define LBM_CASE(L2) \
-    case L2: update_rows<R, L2, sizeof(R) == 4, 1>(u, kc, blk, 0u); break;
+    case L2: update_rows<R, L2, 1>(u, kc, blk, 0u); break;
         LBM_BATCH_LOG2N(LBM_CASE)
 #undef LBM_CASE
     }

@@ -17,26 +17,25 @@ __global__ void __launch_bounds__(MacroThreads<R, LOG2N>::value, MacroThreads<R,
     macro_rows<R, LOG2N, SERIAL, false, RHO64, DIAG>(a, blockIdx.x);
 }
 
-template <typename R, int LOG2N, bool MOMENT_SPACE>
+template <typename R, int LOG2N>
 __global__ void __launch_bounds__(PassThreads<R>::value, PassThreads<R>::min_blocks) update_row_kernel(const __grid_constant__ UpdateArgs<R> a) {
-    update_rows<R, LOG2N, MOMENT_SPACE, 1>(a, a.k, blockIdx.x, 0u);
+    update_rows<R, LOG2N, 1>(a, a.k, blockIdx.x, 0u);
 }
 
 // one row per cluster of CS CTAs (consecutive blockIdx.x)
-template <typename R, int LOG2N, bool MOMENT_SPACE, int CS>
+template <typename R, int LOG2N, int CS>
 __global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(PassThreads<R>::value, PassThreads<R>::min_blocks)
     update_cluster_kernel(const __grid_constant__ UpdateArgs<R> a) {
-    update_rows<R, LOG2N, MOMENT_SPACE, CS>(a, a.k, blockIdx.x / CS, reg::cluster_rank());
+    update_rows<R, LOG2N, CS>(a, a.k, blockIdx.x / CS, reg::cluster_rank());
 }
 
 
 template <typename R, int LOG2N, int CS> static cudaError_t launch_update_cs(const UpdateArgs<R> &a, size_t smem,
                                                                               cudaStream_t s) {
     using F = reg::Line<R, LOG2N, true, CS>;
-    constexpr bool MS = sizeof(R) == 4;  // float32: moment-space collision
     cudaError_t e;
-    if constexpr (CS == 1) e = allow_smem(update_row_kernel<R, LOG2N, MS>);
-    else e = allow_smem(update_cluster_kernel<R, LOG2N, MS, CS>);
+    if constexpr (CS == 1) e = allow_smem(update_row_kernel<R, LOG2N>);
+    else e = allow_smem(update_cluster_kernel<R, LOG2N, CS>);
     if (e != cudaSuccess) return e;
     // the in-kernel row transforms need 6 line buffers per row; refuse a launch without them
     const bool adv = !(a.flags & LBM_FLAG_NO_ADVECTION);
@@ -52,10 +51,10 @@ template <typename R, int LOG2N, int CS> static cudaError_t launch_update_cs(con
     int threads = b.lines_per_batch * F::GL;
     if (threads < nodes) threads = nodes < cap ? ((nodes + 31) & ~31) : cap;
     if constexpr (CS == 1) {
-        update_row_kernel<R, LOG2N, MS><<<a.ny / a.rows, threads, smem, s>>>(b);
+        update_row_kernel<R, LOG2N><<<a.ny / a.rows, threads, smem, s>>>(b);
     } else {
         if (threads < 2 * NF_F + NF_A + NF_M) threads = 2 * NF_F + NF_A + NF_M;  // one prefetching thread per field
-        update_cluster_kernel<R, LOG2N, MS, CS><<<(a.ny / a.rows) * CS, threads, smem, s>>>(b);
+        update_cluster_kernel<R, LOG2N, CS><<<(a.ny / a.rows) * CS, threads, smem, s>>>(b);
     }
     return cudaGetLastError();
 }

@@ -337,6 +337,44 @@ int run_rho64_chain(lbm_ctx *c, const float *fs) {
     return LBM_OK;
 }
 
+void fill_const(const lbm_ctx *c, UpdateConst<float> &k) {
+    for (int i = 0; i < 16; ++i) {
+        const double psi = vel_sq(i) + (i < 4 ? c->p.eta0 * c->p.eta0 : 0.0);
+        k.psi_hi[i] = (float)psi;
+        k.psi_lo[i] = (float)(psi - (double)k.psi_hi[i]);
+    }
+    for (int j = 0; j < 256; ++j) k.minv[j] = (float)c->minv[j];
+}
+// the coefficients of a speed group as the means over its four velocities' images of them
+void fill_const(const lbm_ctx *c, UpdateConst<double> &k) {
+    k.ib = 1.0 / c->p.b;
+    for (int g = 0; g < 4; ++g) {
+        k.psi[g] = vel_sq(4 * g) + (g == 0 ? c->p.eta0 * c->p.eta0 : 0.0);
+        double *o = k.c[g];
+        for (int j = 0; j < 10; ++j) o[j] = 0.0;
+        for (int i = 4 * g; i < 4 * g + 4; ++i) {
+            const double *w = c->minv + i * 16;
+            const double sx = vel_x(i) > 0 ? 1.0 : vel_x(i) < 0 ? -1.0 : 0.0, sy = vel_y(i) > 0 ? 1.0 : vel_y(i) < 0 ? -1.0 : 0.0;
+            o[0] += 0.25 * w[0];
+            o[1] += 0.25 * w[3];
+            o[2] += 0.125 * (w[4] + w[6]);
+            o[3] += 0.125 * (w[13] + w[15]);
+            if (g < 2) {
+                const double s = sx != 0 ? 1.0 : -1.0;
+                o[4] += 0.125 * s * (w[4] - w[6]);
+                o[5] += 0.125 * s * (w[13] - w[15]);
+            } else {
+                o[4] += 0.25 * sx * sy * w[5];
+                o[5] += 0.25 * sx * sy * w[14];
+            }
+            const double wt = g < 2 ? 0.25 : 0.125;  // axis groups: each velocity sees one axis
+            o[6] += wt * (sx * w[1] + sy * w[2]);
+            o[7] += wt * (sx * w[7] + sy * w[8]);
+            o[8] += wt * (sx * w[9] + sy * w[12]);
+            o[9] += wt * (sx * w[11] + sy * w[10]);
+        }
+    }
+}
 template <typename R> UpdateArgs<R> update_args(const lbm_ctx *c, int stage, int rows_per_cta) {
     const lbm_params &p = c->p;
     const bool adv = !(p.flags & LBM_FLAG_NO_ADVECTION);
@@ -358,13 +396,8 @@ template <typename R> UpdateArgs<R> update_args(const lbm_ctx *c, int stage, int
     a.K = (R)p.K;
     a.b = (R)p.b;
     a.eta2 = (R)(p.eta0 * p.eta0);
-    for (int i = 0; i < 16; ++i) {
-        const double psi = vel_sq(i) + (i < 4 ? p.eta0 * p.eta0 : 0.0);
-        a.k.psi_hi[i] = (R)psi;
-        a.k.psi_lo[i] = (R)(psi - (double)a.k.psi_hi[i]);
-    }
     a.flags = p.flags;
-    for (int k = 0; k < 256; ++k) a.k.minv[k] = (R)c->minv[k];
+    fill_const(c, a.k);
     return a;
 }
 

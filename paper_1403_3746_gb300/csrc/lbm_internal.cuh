@@ -262,6 +262,17 @@ template <typename R> struct UpdateConst {
     R psi_hi[16], psi_lo[16];  // psi_i = |v_i|^2 + eta_i^2 as a two-term sum (hi + lo)
     R minv[256];               // inverse of the 16x16 moment matrix, row-major
 };
+// float64: psi of each speed group, and M^-1 reduced by the symmetry of the velocity set. The
+// four velocities of a speed group are images of one another under the reflections of the axes
+// and their exchange, so f^eq of the group is made of one even and two odd sums of moments with
+// common coefficients (update_node64): c[0..3] of rho, E, m_xx + m_yy, psi-m_xx + psi-m_yy; c[4..5] of
+// m_xx - m_yy and its psi partner (axis groups) or m_xy and its psi partner (diagonal groups);
+// c[6..9] of the odd moments j_a, psi-j_a, m_aaa, m_abb along axis a.
+template <> struct UpdateConst<double> {
+    double psi[4];
+    double c[4][10];
+    double ib;  // 1 / b
+};
 template <typename R> struct UpdateArgs {
     const R *fs;     // f of this stage (derivatives, BGK, f^eq moments), [ny][16][nx]
     const R *fbase;  // f^n (the stage starts from it)

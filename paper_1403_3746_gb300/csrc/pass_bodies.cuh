@@ -60,12 +60,9 @@ __device__ __forceinline__ void col_tile(const ColArgs<R> &a, int jobi, int z, i
 // transforms' tables (and register spills) from L1.
 template <typename T> __device__ __forceinline__ T ldcg(const T *p) { return __ldcg(p); }
 
-// a / b in the path's precision: float64 divides exactly; float32 uses the reciprocal unit and
-// one multiply (__fdividef, within 2 ulp for the O(1) physical operands here) instead of the
-// IEEE division sequence.
-template <typename R> __device__ __forceinline__ R quot(R a, R b);
-template <> __device__ __forceinline__ double quot<double>(double a, double b) { return a / b; }
-template <> __device__ __forceinline__ float quot<float>(float a, float b) { return __fdividef(a, b); }
+// a / b in float32: the reciprocal unit and one multiply (__fdividef, within 2 ulp for the O(1)
+// physical operands here) instead of the IEEE division sequence.
+__device__ __forceinline__ float quot(float a, float b) { return __fdividef(a, b); }
 
 // compile-time loop: f(std::integral_constant<int, I>) for I = B .. E-1
 template <int B, int E, class Fn> __device__ __forceinline__ void static_for(Fn &&f) {
@@ -211,10 +208,17 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
         const D divu = dux_dx + duy_dy;
         // van der Waals EOS (Sec. 2.2)
         const D rT = rho * T;
-        const D Pw = quot(D(3) * rT, D(3) - rho) - D(1.125) * rho * rho;
+        D iT2, Pw;
+        if constexpr (sizeof(D) == 8) {  // one division for both quotients
+            const D d3 = D(3) - rho, T2 = T * T, r = D(1) / (d3 * T2);
+            iT2 = d3 * r;
+            Pw = D(3) * rT * (T2 * r) - D(1.125) * rho * rho;
+        } else {
+            iT2 = quot(D(1), T * T);
+            Pw = quot(D(3) * rT, D(3) - rho) - D(1.125) * rho * rho;
+        }
         // Lambda with M = K + H T and grad(M/T) = -K grad T / T^2
         const D Mc = K + H * T;
-        const D iT2 = quot(D(1), T * T);
         const D gx = -K * Tx * iT2, gy = -K * Ty * iT2;
         const D grr = rx * rx + ry * ry;
         const D iso = Mc * (rho * lap + D(0.5) * grr) + rT * (rx * gx + ry * gy);
@@ -293,18 +297,27 @@ template <typename R> struct MomentSums;
 
 template <> struct MomentSums<double> {
     double r = 0, jx = 0, jy = 0, E = 0;
-    __device__ __forceinline__ void add(int i, double f, double psi_hi, double) {
-        r += f;
-        if (vel_x(i) != 0.0) jx += vel_x(i) * f;
-        if (vel_y(i) != 0.0) jy += vel_y(i) * f;
-        E += psi_hi * f;
+    // the four velocities of speed group g, counter-clockwise: opposite pairs enter as sum (to rho
+    // and E) and difference (to j)
+    template <int g> __device__ __forceinline__ void add_group(double f0, double f1, double f2, double f3, double psi) {
+        constexpr double v = vel_x(4 * g);  // the component's magnitude, the same for the group
+        const double s = (f0 + f2) + (f1 + f3), d0 = f0 - f2, d1 = f1 - f3;
+        r += s;
+        E += psi * s;
+        if constexpr (g < 2) {
+            jx += v * d0;
+            jy += v * d1;
+        } else {
+            jx += v * (d0 - d1);
+            jy += v * (d0 + d1);
+        }
     }
-    __device__ __forceinline__ void finish(double b, double &rho, double &ux, double &uy, double &T) const {
+    __device__ __forceinline__ void finish(double ib, double &rho, double &ux, double &uy, double &T) const {
         rho = r;
         const double ir = 1.0 / r;
         ux = jx * ir;
         uy = jy * ir;
-        T = (E * ir - (ux * ux + uy * uy)) / b;
+        T = (E * ir - (ux * ux + uy * uy)) * ib;
     }
 };
 
@@ -453,9 +466,9 @@ __host__ __device__ constexpr bool mom_odd(int j) { return (mom_px(j) + mom_py(j
 
 // One node (y, x) of the fused update pass: the body of its node loop. dl: the node's row of
 // d_x line buffers (line q at dl + q ls, natural order), xl: the node's index in them.
-template <typename R, int LOG2N, bool MOMENT_SPACE, bool AX_POSSIBLE>
-__device__ __forceinline__ void update_node(const UpdateArgs<R> &a, const UpdateConst<R> &kc, size_t y, int x,
-                                            const reg::C<R> *dl, size_t ls, int xl) {
+template <typename R, int LOG2N>
+__device__ __forceinline__ void update_node32(const UpdateArgs<R> &a, const UpdateConst<R> &kc, size_t y, int x,
+                                              const reg::C<R> *dl, size_t ls, int xl) {
     using CT = reg::C<R>;
     constexpr int NX = 1 << LOG2N;
     const R b = a.b, K = a.K, tau_inv = a.tau_inv, h = a.h;
@@ -464,7 +477,6 @@ __device__ __forceinline__ void update_node(const UpdateArgs<R> &a, const Update
     const bool frc = !(a.flags & LBM_FLAG_NO_FORCE);
     const bool same_base = a.fbase == a.fs;
     const bool iso = a.flags & LBM_FLAG_ISOTHERMAL;
-    const bool ax_mode = AX_POSSIBLE && a.Ax != nullptr;
     {
         const R *fn = a.fs + y * NF_F * NX + x;       // field i at fn[i * NX]
         const R *an = a.Ay + y * NF_A * NX + x;       // slot k at an[k * NX]
@@ -507,12 +519,8 @@ __device__ __forceinline__ void update_node(const UpdateArgs<R> &a, const Update
                 // row line's second field has the opposite v_x, hence the sign of its part)
                 constexpr int xs = xslot(i), ys = yslot(i);
                 if constexpr (xs >= 0) {
-                    if (ax_mode) {
-                        dfo = -h * (R(vel_x(i)) * ldcg(a.Ax + (y * NF_F + i) * NX + x));
-                    } else {
-                        const CT d = dl[(xs >> 1) * ls + xl];
-                        dfo = (xs & 1) ? -d.y : d.x;
-                    }
+                    const CT d = dl[(xs >> 1) * ls + xl];
+                    dfo = (xs & 1) ? -d.y : d.x;
                 }
                 if constexpr (ys >= 0) dfo += ldcg(an + ys * NX);
             }
@@ -521,82 +529,63 @@ __device__ __forceinline__ void update_node(const UpdateArgs<R> &a, const Update
             return (same_base ? fsv[i] : ldcg(bn + i * NX)) + dfo;
         };
         MomentSums<R> acc;
-        if constexpr (MOMENT_SPACE) {
-            // neq = M^-1 (m^eq - M f) over the 12 non-conserved moments only (the 4 conserved
-            // ones agree exactly), so the rounding of M^-1 to float32 cannot bias mass, momentum
-            // or energy: its error scales with the non-equilibrium part instead of with rho.
-            // Opposite-velocity pairs: even moments see fi + fk, odd ones fi - fk, and
-            // ne_i, ne_k = E +- O from the even and odd columns of M^-1.
-            R sp[8], dp[8];
+        // neq = M^-1 (m^eq - M f) over the 12 non-conserved moments only (the 4 conserved
+        // ones agree exactly), so the rounding of M^-1 to float32 cannot bias mass, momentum
+        // or energy: its error scales with the non-equilibrium part instead of with rho.
+        // Opposite-velocity pairs: even moments see fi + fk, odd ones fi - fk, and
+        // ne_i, ne_k = E +- O from the even and odd columns of M^-1.
+        R sp[8], dp[8];
+        static_for<0, 8>([&](auto P) {
+            constexpr int p = decltype(P)::value, i = pair_rep(p);
+            sp[p] = fsv[i] + fsv[i + 2];
+            dp[p] = fsv[i] - fsv[i + 2];
+        });
+        const R eta2 = a.eta2;
+        R dm[12];
+        static_for<0, 12>([&](auto J) {
+            constexpr int j = decltype(J)::value;
+            R mf = 0, me = 0;
             static_for<0, 8>([&](auto P) {
                 constexpr int p = decltype(P)::value, i = pair_rep(p);
-                sp[p] = fsv[i] + fsv[i + 2];
-                dp[p] = fsv[i] - fsv[i + 2];
+                const R g = mom_odd(j) ? dp[p] : sp[p];
+                if constexpr (mom_entry(j, i) != 0.0) mf += R(mom_entry(j, i)) * g;
+                if constexpr (mom_entry_eta(j, i) != 0.0) me += R(mom_entry_eta(j, i)) * g;
             });
-            const R eta2 = a.eta2;
-            R dm[12];
+            dm[j] = m[4 + j] - (mf + eta2 * me);
+        });
+        // isothermal: the energy moment (row 3, even) is not conserved by the thermostat either
+        R dE = 0;
+        if (iso) {
+            R me = 0;
+            static_for<0, 8>([&](auto P) {
+                constexpr int p = decltype(P)::value;
+                me += kc.psi_hi[pair_rep(p)] * sp[p];
+            });
+            dE = m[3] - me;
+        }
+        static_for<0, 8>([&](auto P) {
+            constexpr int p = decltype(P)::value, i = pair_rep(p);
+            R ev = 0, od = 0;
             static_for<0, 12>([&](auto J) {
                 constexpr int j = decltype(J)::value;
-                R mf = 0, me = 0;
-                static_for<0, 8>([&](auto P) {
-                    constexpr int p = decltype(P)::value, i = pair_rep(p);
-                    const R g = mom_odd(j) ? dp[p] : sp[p];
-                    if constexpr (mom_entry(j, i) != 0.0) mf += R(mom_entry(j, i)) * g;
-                    if constexpr (mom_entry_eta(j, i) != 0.0) me += R(mom_entry_eta(j, i)) * g;
-                });
-                dm[j] = m[4 + j] - (mf + eta2 * me);
+                if constexpr (!minv_zero(i, j)) {
+                    if constexpr (mom_odd(j)) od += kc.minv[i * 16 + 4 + j] * dm[j];
+                    else ev += kc.minv[i * 16 + 4 + j] * dm[j];
+                }
             });
-            // isothermal: the energy moment (row 3, even) is not conserved by the thermostat either
-            R dE = 0;
-            if (iso) {
-                R me = 0;
-                static_for<0, 8>([&](auto P) {
-                    constexpr int p = decltype(P)::value;
-                    me += kc.psi_hi[pair_rep(p)] * sp[p];
-                });
-                dE = m[3] - me;
+            if (iso) ev += kc.minv[i * 16 + 3] * dE;
+            R qe = 0, qo = 0;
+            if (frc) {
+                qe = hal + hcc * R(vel_sq(i));
+                if constexpr (vel_x(i) != 0.0) qo += hbx * R(vel_x(i));
+                if constexpr (vel_y(i) != 0.0) qo += hby * R(vel_y(i));
             }
-            static_for<0, 8>([&](auto P) {
-                constexpr int p = decltype(P)::value, i = pair_rep(p);
-                R ev = 0, od = 0;
-                static_for<0, 12>([&](auto J) {
-                    constexpr int j = decltype(J)::value;
-                    if constexpr (!minv_zero(i, j)) {
-                        if constexpr (mom_odd(j)) od += kc.minv[i * 16 + 4 + j] * dm[j];
-                        else ev += kc.minv[i * 16 + 4 + j] * dm[j];
-                    }
-                });
-                if (iso) ev += kc.minv[i * 16 + 3] * dE;
-                R qe = 0, qo = 0;
-                if (frc) {
-                    qe = hal + hcc * R(vel_sq(i));
-                    if constexpr (vel_x(i) != 0.0) qo += hbx * R(vel_x(i));
-                    if constexpr (vel_y(i) != 0.0) qo += hby * R(vel_y(i));
-                }
-                const R fi = out_value(std::integral_constant<int, i>{}, ev + od, qe + qo);
-                const R fk = out_value(std::integral_constant<int, i + 2>{}, ev - od, qe - qo);
-                on[i * NX] = fi;
-                on[(i + 2) * NX] = fk;
-                acc.template add_pair<i>(fi, fk, kc.psi_hi[i], kc.psi_lo[i]);
-            });
-        } else {
-            // float64: f^eq = M^-1 m^eq directly
-            static_for<0, 16>([&](auto I) {
-                constexpr int i = decltype(I)::value;
-                R fe = 0;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) fe += kc.minv[i * 16 + j] * m[j];
-                R q = 0;
-                if (frc) {
-                    q = hal + hcc * R(vel_sq(i));
-                    if constexpr (vel_x(i) != 0.0) q += hbx * R(vel_x(i));
-                    if constexpr (vel_y(i) != 0.0) q += hby * R(vel_y(i));
-                }
-                const R fo = out_value(I, fe - fsv[i], q);
-                on[i * NX] = fo;
-                acc.add(i, fo, kc.psi_hi[i], kc.psi_lo[i]);
-            });
-        }
+            const R fi = out_value(std::integral_constant<int, i>{}, ev + od, qe + qo);
+            const R fk = out_value(std::integral_constant<int, i + 2>{}, ev - od, qe - qo);
+            on[i * NX] = fi;
+            on[(i + 2) * NX] = fk;
+            acc.template add_pair<i>(fi, fk, kc.psi_hi[i], kc.psi_lo[i]);
+        });
         R nr, nux, nuy, nT;
         acc.finish(b, nr, nux, nuy, nT);
         if (iso) nT = a.T_iso;
@@ -607,11 +596,109 @@ __device__ __forceinline__ void update_node(const UpdateArgs<R> &a, const Update
     }
 }
 
+// The float64 node. It is bound by the 2 float64 operations per clock and SM, so it is written
+// for their number: f^eq by speed groups from the symmetry-reduced M^-1 (UpdateConst<double>: 84
+// operations instead of the 256 of the full matrix), forcing factors and moment sums by opposite
+// pairs, one reciprocal for 1/(rho T), 1/(rho T^2). About 310 operations per node instead of 570:
+// 1024^2 update pass 1.58 -> 1.10 ms per launch (row transforms included).
+template <int LOG2N, bool AX_POSSIBLE>
+__device__ __forceinline__ void update_node64(const UpdateArgs<double> &a, const UpdateConst<double> &kc, size_t y, int x,
+                                              const double2 *dl, size_t ls, int xl) {
+    constexpr int NX = 1 << LOG2N;
+    const double K = a.K, h = a.h;
+    const bool adv = !(a.flags & LBM_FLAG_NO_ADVECTION);
+    const bool col = !(a.flags & LBM_FLAG_NO_COLLISION);
+    const bool frc = !(a.flags & LBM_FLAG_NO_FORCE);
+    const bool same_base = a.fbase == a.fs;
+    const bool ax_mode = AX_POSSIBLE && a.Ax != nullptr;
+    const double *fn = a.fs + y * NF_F * NX + x, *an = a.Ay + y * NF_A * NX + x, *bn = a.fbase + y * NF_F * NX + x;
+    double *mn = a.m + y * NF_M * NX + x, *on = a.fout + y * NF_F * NX + x;
+    const double rho = ldcg(mn + M_RHO * NX), ux = ldcg(mn + M_UX * NX), uy = ldcg(mn + M_UY * NX);
+    const double T = ldcg(mn + M_T * NX);
+    const double xx = ux * ux, yy = uy * uy, u2 = xx + yy;
+    // I_i = -(al + bx v_ix + by v_iy + cc |v_i|^2) f_i^eq, h folded in (as in update_node32)
+    double hal = 0, hbx = 0, hby = 0, hcc = 0;
+    if (frc) {
+        const double irT = 1.0 / (rho * T), irTT = irT * (irT * rho);  // 1 / (rho T), 1 / (rho T^2)
+        const double hB = h * irT, hC = h * irTT;
+        const double Bx = (ldcg(mn + M_DSXX * NX) + ldcg(mn + M_DSXYY * NX)) * hB;
+        const double By = (ldcg(mn + M_DSXY * NX) + ldcg(mn + M_DSYY * NX)) * hB;
+        const double C = ldcg(mn + M_CNUM * NX) - K * rho * ldcg(mn + M_RY * NX) * ldcg(mn + M_DDIVUY * NX);
+        hcc = (0.5 * C + (ldcg(mn + M_DQX * NX) + ldcg(mn + M_DQY * NX))) * hC;
+        const double cc2 = 2.0 * hcc;
+        hal = hcc * (u2 - 2.0 * T) - Bx * ux - By * uy;
+        hbx = Bx - cc2 * ux;
+        hby = By - cc2 * uy;
+    }
+    const double htau = h * a.tau_inv;
+    // moments of f^eq: even ones as sums and differences of the xx and yy parts, odd ones per axis
+    const double e = (a.b + 2.0) * T + u2, gq = (a.b + 4.0) * T + u2;
+    const double jx = rho * ux, jy = rho * uy, rd = rho * (xx - yy), rxy = jx * uy;
+    const double mE = rho * (a.b * T + u2), mS = rho * (2.0 * T + u2), mP = rho * (2.0 * T * e + gq * u2);
+    const double mD = rd, mQ = gq * rd, mXY = rxy, mPXY = gq * rxy;
+    const double ox[4] = {jx, jx * e, jx * (3.0 * T + xx), jx * (T + yy)};
+    const double oy[4] = {jy, jy * e, jy * (3.0 * T + yy), jy * (T + xx)};
+    MomentSums<double> acc;
+    static_for<0, 4>([&](auto GI) {
+        constexpr int g = decltype(GI)::value;
+        constexpr double v = vel_x(4 * g), v2 = vel_sq(4 * g);
+        const double *c = kc.c[g];
+        const double ev = c[0] * rho + c[1] * mE + c[2] * mS + c[3] * mP;
+        const double ed = g < 2 ? c[4] * mD + c[5] * mQ : c[4] * mXY + c[5] * mPXY;
+        const double odx = c[6] * ox[0] + c[7] * ox[1] + c[8] * ox[2] + c[9] * ox[3];
+        const double ody = c[6] * oy[0] + c[7] * oy[1] + c[8] * oy[2] + c[9] * oy[3];
+        // even and odd parts of the pairs (0, 2) and (1, 3): axis groups x and y, diagonal groups
+        // (+,+) and (-,+)
+        const double e0 = ev + ed, e1 = ev - ed;
+        const double o0 = g < 2 ? odx : ody + odx, o1 = g < 2 ? ody : ody - odx;
+        const double qe = hal + hcc * v2;
+        const double q0 = g < 2 ? v * hbx : v * (hby + hbx), q1 = g < 2 ? v * hby : v * (hby - hbx);
+        double out[4];
+        static_for<0, 4>([&](auto KI) {
+            constexpr int k = decltype(KI)::value, i = 4 * g + k, xs = xslot(i), ys = yslot(i);
+            const double ee = k & 1 ? e1 : e0, oo = k & 1 ? o1 : o0, qq = k & 1 ? q1 : q0;
+            const double fe = k < 2 ? ee + oo : ee - oo, q = k < 2 ? qe + qq : qe - qq;
+            const double f = ldcg(fn + i * NX);
+            double dfo = 0;  // h R_i
+            if (adv) {
+                if constexpr (xs >= 0) {
+                    if (ax_mode) {
+                        dfo = -h * (vel_x(i) * ldcg(a.Ax + (y * NF_F + i) * NX + x));
+                    } else {
+                        const double2 d = dl[(xs >> 1) * ls + xl];
+                        dfo = (xs & 1) ? -d.y : d.x;
+                    }
+                }
+                if constexpr (ys >= 0) dfo += ldcg(an + ys * NX);
+            }
+            if (col) dfo += htau * (fe - f);
+            if (frc) dfo -= q * fe;
+            out[k] = (same_base ? f : ldcg(bn + i * NX)) + dfo;
+            on[i * NX] = out[k];
+        });
+        acc.template add_group<g>(out[0], out[1], out[2], out[3], kc.psi[g]);
+    });
+    double nr, nux, nuy, nT;
+    acc.finish(kc.ib, nr, nux, nuy, nT);
+    if (a.flags & LBM_FLAG_ISOTHERMAL) nT = a.T_iso;
+    mn[M_RHO * NX] = nr;
+    mn[M_UX * NX] = nux;
+    mn[M_UY * NX] = nuy;
+    mn[M_T * NX] = nT;
+}
+
+template <typename R, int LOG2N, bool AX_POSSIBLE>
+__device__ __forceinline__ void update_node(const UpdateArgs<R> &a, const UpdateConst<R> &kc, size_t y, int x,
+                                            const reg::C<R> *dl, size_t ls, int xl) {
+    if constexpr (sizeof(R) == 8) update_node64<LOG2N, AX_POSSIBLE>(a, kc, y, x, dl, ls, xl);
+    else update_node32<R, LOG2N>(a, kc, y, x, dl, ls, xl);
+}
+
 // CS = 1: a CTA owns `rows` whole rows. CS > 1 (float32 rows of 2048 or more, 4096 for CS = 4, one row per
 // cluster): the CS CTAs of a cluster split the row's line transforms (fft_reg.cuh) and CTA
 // `rank` runs the node loop over its x-range [rank N/CS, (rank + 1) N/CS), whose derivatives the
 // transforms leave in its own shared memory.
-template <typename R, int LOG2N, bool MOMENT_SPACE, int CS>
+template <typename R, int LOG2N, int CS>
 __device__ __forceinline__ void update_rows(const UpdateArgs<R> &a, const UpdateConst<R> &kc, int blk, unsigned rank) {
     using F = reg::Line<R, LOG2N, true, CS>;
     using CT = typename F::CT;
@@ -682,8 +769,7 @@ __device__ __forceinline__ void update_rows(const UpdateArgs<R> &a, const Update
 
     for (int idx = threadIdx.x; idx < nodes; idx += blockDim.x) {
         const int r = idx / NL, xl = idx % NL;  // xl: index in this CTA's line buffers
-        update_node<R, LOG2N, MOMENT_SPACE, AX_POSSIBLE>(a, kc, (size_t)(y0 + r), x0 + xl, sb + (size_t)r * SM,
-                                                         (size_t)NR * SM, xl);
+        update_node<R, LOG2N, AX_POSSIBLE>(a, kc, (size_t)(y0 + r), x0 + xl, sb + (size_t)r * SM, (size_t)NR * SM, xl);
     }
 }
 
