@@ -190,7 +190,7 @@ __global__ void field_out_kernel(const R *src, int ld, double *out, int nx, int 
 // per CTA, G threads per line (fft_reg.cuh); row y of every field at + y * ld. A field may be
 // transformed in place (out = in): every thread reads its points before any is written back.
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(MaxThreads<R>::value) row_deriv_kernel(const __grid_constant__ RowDerivArgs<R> a) {
+__global__ void __launch_bounds__(MaxThreads<R>::value, MaxThreads<R>::min_blocks) row_deriv_kernel(const __grid_constant__ RowDerivArgs<R> a) {
     using F = reg::Line<R, LOG2N, false>;
     using CT = typename F::CT;
     constexpr int G = F::G, E = F::E;

@@ -18,13 +18,13 @@ __global__ void __launch_bounds__(MacroThreads<R, LOG2N>::value, MacroThreads<R,
 }
 
 template <typename R, int LOG2N>
-__global__ void __launch_bounds__(PassThreads<R>::value, PassThreads<R>::min_blocks) update_row_kernel(const __grid_constant__ UpdateArgs<R> a) {
+__global__ void __launch_bounds__(UpdateThreads<R, LOG2N>::value, UpdateThreads<R, LOG2N>::min_blocks) update_row_kernel(const __grid_constant__ UpdateArgs<R> a) {
     update_rows<R, LOG2N, 1>(a, a.k, blockIdx.x, 0u);
 }
 
 // one row per cluster of CS CTAs (consecutive blockIdx.x)
 template <typename R, int LOG2N, int CS>
-__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(PassThreads<R>::value, PassThreads<R>::min_blocks)
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(UpdateThreads<R, LOG2N>::value, UpdateThreads<R, LOG2N>::min_blocks)
     update_cluster_kernel(const __grid_constant__ UpdateArgs<R> a) {
     update_rows<R, LOG2N, CS>(a, a.k, blockIdx.x / CS, reg::cluster_rank());
 }
@@ -44,7 +44,7 @@ template <typename R, int LOG2N, int CS> static cudaError_t launch_update_cs(con
     if (a.Ax != nullptr && !(sizeof(R) == 8 && LOG2N == 12 && CS == 1)) return cudaErrorInvalidValue;
     if (CS > 1 && a.rows != 1) return cudaErrorInvalidValue;
     // LB line transforms at a time; at least one thread per node of the CTA's rows (up to the cap)
-    constexpr int cap = PassThreads<R>::value;
+    constexpr int cap = UpdateThreads<R, LOG2N>::value;
     UpdateArgs<R> b = a;
     b.lines_per_batch = update_lines_per_batch(6 * a.rows, F::GL, cap);
     const int nodes = a.rows * F::NL;

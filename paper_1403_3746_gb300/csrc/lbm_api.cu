@@ -871,11 +871,11 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
     // launch geometry
     int smem_optin = 0;
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-    pass_geometry(nx, ny, c->fsize, &c->geo);
+    pass_geometry(nx, ny, c->fsize, &c->geo, nb);
     size_t need =
         std::max(std::max(c->geo.upd_smem, c->geo.macro_smem), std::max(c->geo.col_smem, c->geo.rowd_smem));  // flux = col
     if (c->rho64) {  // the density chain's float64 column and row transforms
-        pass_geometry(nx, ny, 8, &c->geo64);
+        pass_geometry(nx, ny, 8, &c->geo64, nb);
         need = std::max(need, std::max(c->geo64.col_smem, c->geo64.rowd_smem));
     }
     if (need > (size_t)smem_optin) {
@@ -2399,7 +2399,7 @@ void filter_table(int N, double alpha, double p, double *kf) {
     }
 }
 
-void pass_geometry(int nx, int ny, size_t esize, Geometry *g) {
+void pass_geometry(int nx, int ny, size_t esize, Geometry *g, int nb) {
     int lx = 0, ly = 0;
     while ((1 << lx) < nx) ++lx;
     while ((1 << ly) < ny) ++ly;
@@ -2424,6 +2424,10 @@ void pass_geometry(int nx, int ny, size_t esize, Geometry *g) {
     int r0 = 512 / nx;
     if (r0 < 1) r0 = 1;
     if (r0 > ny) r0 = ny;
+    // float64 nodes are bound by each SM's own float64 unit: fewer rows per CTA until there is a CTA
+    // for each of the 152 SMs (64^2: 8 rows -> 1, update pass 67 -> 35 us per launch; float32 passes of
+    // small grids are bound by latency and gained nothing)
+    while (esize == 8 && r0 > 1 && (long long)ny * nb / r0 < 152) r0 >>= 1;
     int r = r0;
     while (r > 1 && 6 * r * SM > 200 * 1024) r >>= 1;  // update: 6 line buffers per row
     g->rows_upd = r;

@@ -59,19 +59,28 @@ __host__ __device__ constexpr int yslot(int i) { return i < 8 ? ((i & 1) ? i / 2
 __host__ __device__ constexpr int line_E(int log2n) { return log2n < 4 ? (1 << log2n) : 16; }
 __host__ __device__ constexpr int line_G(int log2n) { return (1 << log2n) / line_E(log2n); }
 __host__ __device__ constexpr int line_smem(int log2n) { return (1 << log2n) + ((1 << log2n) >> 4) + 2; }
-// threads per CTA of the line-transform kernels: float32 768 (<= 85 registers per thread),
-// float64 384 (<= 170): one line's 16 complex points live in registers
+// threads per CTA of the line-transform kernels (one line's 16 complex points per thread live in
+// registers): float32 768 (<= 85 registers per thread); float64 256, two CTAs resident per SM (<=
+// 128 registers). The fixed-point passes are bound by issue and latency: at 168 registers one CTA
+// of 256 threads left 8 warps per SM (1024^2: column pass 524 -> 322 us per launch, flux 160 -> 100,
+// macro 480 -> 416, update 1.10 -> 1.01 ms).
 template <typename R> struct MaxThreads {
-    static constexpr int value = sizeof(R) == 8 ? 384 : 768;
+    static constexpr int value = sizeof(R) == 8 ? 256 : 768;
+    static constexpr int min_blocks = sizeof(R) == 8 ? 2 : 1;
 };
-__host__ __device__ constexpr int max_threads(size_t esize) { return esize == 8 ? 384 : 768; }
+__host__ __device__ constexpr int max_threads(size_t esize) { return esize == 8 ? 256 : 768; }
 // column and update kernels: float32 CTAs of at most 512 threads, two resident per SM
-// (<= 64 registers per thread); float64 as above
+// (<= 64 registers per thread); float64 as above, but the update pass of rows of 2048 and more,
+// whose line buffers leave one CTA per SM, takes 384 threads
 template <typename R> struct PassThreads {
-    static constexpr int value = sizeof(R) == 8 ? 384 : 512;
-    static constexpr int min_blocks = sizeof(R) == 8 ? 1 : 2;
+    static constexpr int value = sizeof(R) == 8 ? 256 : 512;
+    static constexpr int min_blocks = 2;
 };
-__host__ __device__ constexpr int pass_threads(size_t esize) { return esize == 8 ? 384 : 512; }
+__host__ __device__ constexpr int pass_threads(size_t esize) { return esize == 8 ? 256 : 512; }
+template <typename R, int LOG2N> struct UpdateThreads {
+    static constexpr bool wide = sizeof(R) == 8 && LOG2N >= 11;
+    static constexpr int value = wide ? 384 : PassThreads<R>::value, min_blocks = wide ? 1 : 2;
+};
 // CTAs per cluster for a column tile of W columns of lines of 2^log2n points: 1 when the tile's
 // W/2 lines fit one CTA's threads, else the split (2 or 4, lines of 512+ points) that makes
 // them fit; 0 when no split serves the width
@@ -123,11 +132,11 @@ __host__ __device__ constexpr size_t col_smem(int W, int log2n, size_t esize) {
 // step 1.70 -> 1.56 ms against one); at 512 (nx = 4096) one (two at 64 registers spill, and
 // that macro pass took 620 instead of 535 us per launch at 4096^2)
 __host__ __device__ constexpr int macro_threads(size_t esize, int log2n) {
-    return esize == 8 ? 384 : (2 * line_G(log2n) > 128 ? 2 * line_G(log2n) : 128);
+    return esize == 8 ? 256 : (2 * line_G(log2n) > 128 ? 2 * line_G(log2n) : 128);
 }
 template <typename R, int LOG2N> struct MacroThreads {
     static constexpr int value = macro_threads(sizeof(R), LOG2N);
-    static constexpr int min_blocks = sizeof(R) == 8 ? 1 : value == 128 ? 7 : value == 256 ? 3 : 1;
+    static constexpr int min_blocks = sizeof(R) == 8 ? 2 : value == 128 ? 7 : value == 256 ? 3 : 1;
 };
 // every supported line length 2^1 .. 2^12
 #define LBM_FOR_LOG2N(X) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12)
@@ -165,7 +174,8 @@ struct Geometry {
     int col_kind = 0;           // column pass: LBM_COL_DIRECT, LBM_COL_TMA, LBM_COL_LOOKAHEAD or LBM_COL_TMA1 (width colW)
     int flux_kind = 0;          // flux column pass: the same choice (width fluxW)
 };
-void pass_geometry(int nx, int ny, size_t esize, Geometry *g);
+// nb: instances stacked along y
+void pass_geometry(int nx, int ny, size_t esize, Geometry *g, int nb = 1);
 
 // ---- HBM layout ------------------------------------------------------------------------
 // Row-interleaved field blocks: a group of NF fields over an nx x ny grid is stored as
