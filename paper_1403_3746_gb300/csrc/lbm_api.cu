@@ -6,6 +6,7 @@
 // instance from grid.z. A batch (lbm_batch_*) groups instances of different sizes into
 // contexts, one per size, whose steps run as parallel branches of one CUDA graph.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -2367,7 +2368,9 @@ void fixed_twiddles(int N, longlong2 *out) {
             const int q = a / (2 * O), b = a % (2 * O);  // quadrant and angle within it
             const long long x = b <= O ? c[b] : s[2 * O - b], y = b <= O ? s[b] : c[2 * O - b];
             const long long re = q == 0 ? x : q == 1 ? -y : q == 2 ? -x : y, im = q == 0 ? y : q == 1 ? x : q == 2 ? -y : -x;
-            r[a] = longlong2{fixed::balance(re), fixed::balance(-im)};
+            // (a low half of -2^31, which has no negative, is moved by one unit)
+            auto root = [](long long w) { return fixed::balance(fixed::lo32(w) == INT_MIN ? w + 1 : w); };
+            r[a] = longlong2{root(re), root(-im)};
         }
         return r;
     }();
