@@ -14,7 +14,7 @@ namespace lbm {
 
 template <typename R, int LOG2N, bool SERIAL, bool RHO64, bool DIAG = false>
 __global__ void __launch_bounds__(MacroThreads<R, LOG2N>::value, MacroThreads<R, LOG2N>::min_blocks) macro_row_kernel(const __grid_constant__ MacroArgs<R> a) {
-    macro_rows<R, LOG2N, SERIAL, false, RHO64, DIAG>(a, blockIdx.x);
+    macro_rows<R, LOG2N, SERIAL, macro_extra(LOG2N), RHO64, DIAG>(a, blockIdx.x);
 }
 
 template <typename R, int LOG2N>
@@ -77,12 +77,13 @@ template <typename R, int LOG2N> static cudaError_t launch_macro_n(const MacroAr
     // three line buffers per row; refuse less
     const size_t need = (size_t)3 * a.rows * F::STRIDE * sizeof(typename F::CT);
     if (smem < need) return cudaErrorInvalidValue;
+    const int threads = macro_cta_threads(a.rows, LOG2N, sizeof(R), a.serial);
     if constexpr (sizeof(R) == 8 && LOG2N == 12) {  // the only shape that needs the serial form
         if (a.serial) {
             if (a.r64) return cudaErrorInvalidValue;
             cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, true, false>);
             if (e != cudaSuccess) return e;
-            macro_row_kernel<R, LOG2N, true, false><<<a.ny / a.rows, a.rows * F::G, smem, s>>>(a);
+            macro_row_kernel<R, LOG2N, true, false><<<a.ny / a.rows, threads, smem, s>>>(a);
             return cudaGetLastError();
         }
     }
@@ -92,7 +93,7 @@ template <typename R, int LOG2N> static cudaError_t launch_macro_n(const MacroAr
         if (a.diag_partial) {  // the diagnostics of the input state fused in
             cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, false, true>);
             if (e != cudaSuccess) return e;
-            macro_row_kernel<R, LOG2N, false, false, true><<<a.ny / a.rows, 2 * a.rows * F::G, smem, s>>>(a);
+            macro_row_kernel<R, LOG2N, false, false, true><<<a.ny / a.rows, threads, smem, s>>>(a);
             return cudaGetLastError();
         }
     }
@@ -100,14 +101,14 @@ template <typename R, int LOG2N> static cudaError_t launch_macro_n(const MacroAr
         if (a.r64) {
             cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, true>);
             if (e != cudaSuccess) return e;
-            macro_row_kernel<R, LOG2N, false, true><<<a.ny / a.rows, 2 * a.rows * F::G, smem, s>>>(a);
+            macro_row_kernel<R, LOG2N, false, true><<<a.ny / a.rows, threads, smem, s>>>(a);
             return cudaGetLastError();
         }
     }
     if (a.r64) return cudaErrorInvalidValue;
     cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, false>);
     if (e != cudaSuccess) return e;
-    macro_row_kernel<R, LOG2N, false, false><<<a.ny / a.rows, 2 * a.rows * F::G, smem, s>>>(a);
+    macro_row_kernel<R, LOG2N, false, false><<<a.ny / a.rows, threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -1733,7 +1733,7 @@ int lbm_launch_plan(int nx, int ny, int precision, int out[18]) {
     Geometry g;
     pass_geometry(nx, ny, es, &g);
     const int v[18] = {g.colW, (g.colW / 2) * line_G(ly) / std::max(1, col_cluster(g.colW, ly, es)), (int)g.col_smem,
-                       g.rows_macro, g.rows_macro * line_G(lx) * (g.macro_serial ? 1 : 2), (int)g.macro_smem,
+                       g.rows_macro, macro_cta_threads(g.rows_macro, lx, es, g.macro_serial), (int)g.macro_smem,
                        g.macro_serial ? 1 : 0,
                        g.rows_upd, (int)g.upd_smem, g.upd_ax ? 1 : 0,
                        g.rows_rowd, g.rows_rowd * line_G(lx), (int)g.rowd_smem,

@@ -134,6 +134,17 @@ __host__ __device__ constexpr size_t col_smem(int W, int log2n, size_t esize) {
 __host__ __device__ constexpr int macro_threads(size_t esize, int log2n) {
     return esize == 8 ? 256 : (2 * line_G(log2n) > 128 ? 2 * line_G(log2n) : 128);
 }
+// threads of a macro CTA: the two lines of each row, and for rows of up to 512 nodes a thread per node
+// as far as the bound goes (the threads beyond the lines only keep the barriers while those are
+// transformed): with the 2 G threads of a row's lines alone each ran 8 nodes one after another
+__host__ __device__ constexpr bool macro_extra(int log2n) { return log2n <= 9; }
+__host__ __device__ constexpr int macro_cta_threads(int rows, int log2n, size_t esize, bool serial) {
+    const int lines = rows * line_G(log2n) * (serial ? 1 : 2);
+    if (!macro_extra(log2n)) return lines;
+    const int nodes = ((rows << log2n) + 31) & ~31, cap = macro_threads(esize, log2n);
+    const int want = nodes < cap ? nodes : cap;
+    return want > lines ? want : lines;
+}
 template <typename R, int LOG2N> struct MacroThreads {
     static constexpr int value = macro_threads(sizeof(R), LOG2N);
     static constexpr int min_blocks = sizeof(R) == 8 ? 2 : value == 128 ? 7 : value == 256 ? 3 : 1;

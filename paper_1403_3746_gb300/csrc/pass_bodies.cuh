@@ -172,7 +172,7 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
     using D = std::conditional_t<RHO64, double, R>;  // type of the rho-dependent terms
     const D K = RHO64 ? (D)a.K64 : (D)a.K, H = RHO64 ? (D)a.H64 : (D)a.H, q = RHO64 ? (D)a.q64 : (D)a.q,
             zeta = RHO64 ? (D)a.zeta64 : (D)a.zeta;
-    static_assert(!DIAG || (sizeof(R) == 4 && !RHO64 && !SERIAL && !EXTRA), "fused diagnostics: float32 pass only");
+    static_assert(!DIAG || (sizeof(R) == 4 && !RHO64 && !SERIAL), "fused diagnostics: float32 pass only");
     FPair dS[DIAG ? 5 : 1];
     for (int idx = threadIdx.x; idx < nodes; idx += blockDim.x) {
         const int rr = idx / NX, x = idx % NX;
