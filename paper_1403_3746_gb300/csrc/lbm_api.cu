@@ -346,34 +346,41 @@ void fill_const(const lbm_ctx *c, UpdateConst<float> &k) {
     }
     for (int j = 0; j < 256; ++j) k.minv[j] = (float)c->minv[j];
 }
-// the coefficients of a speed group as the means over its four velocities' images of them
+// the coefficients of a speed group: the means over its four velocities' images of the entries of
+// M^-1 (w[j]: of moment j), then collected by powers of T, u^2 and d
 void fill_const(const lbm_ctx *c, UpdateConst<double> &k) {
-    k.ib = 1.0 / c->p.b;
+    const double b = c->p.b;
+    k.ib = 1.0 / b;
+    k.b4 = b + 4.0;
+    k.b24 = 2.0 * b + 4.0;
+    k.b6 = b + 6.0;
     for (int g = 0; g < 4; ++g) {
         k.psi[g] = vel_sq(4 * g) + (g == 0 ? c->p.eta0 * c->p.eta0 : 0.0);
-        double *o = k.c[g];
-        for (int j = 0; j < 10; ++j) o[j] = 0.0;
+        double one = 0, en = 0, s2 = 0, s4 = 0, d2 = 0, d4 = 0, j = 0, pj = 0, aaa = 0, abb = 0;
         for (int i = 4 * g; i < 4 * g + 4; ++i) {
             const double *w = c->minv + i * 16;
             const double sx = vel_x(i) > 0 ? 1.0 : vel_x(i) < 0 ? -1.0 : 0.0, sy = vel_y(i) > 0 ? 1.0 : vel_y(i) < 0 ? -1.0 : 0.0;
-            o[0] += 0.25 * w[0];
-            o[1] += 0.25 * w[3];
-            o[2] += 0.125 * (w[4] + w[6]);
-            o[3] += 0.125 * (w[13] + w[15]);
+            one += 0.25 * w[0];
+            en += 0.25 * w[3];
+            s2 += 0.125 * (w[4] + w[6]);
+            s4 += 0.125 * (w[13] + w[15]);
             if (g < 2) {
                 const double s = sx != 0 ? 1.0 : -1.0;
-                o[4] += 0.125 * s * (w[4] - w[6]);
-                o[5] += 0.125 * s * (w[13] - w[15]);
+                d2 += 0.125 * s * (w[4] - w[6]);
+                d4 += 0.125 * s * (w[13] - w[15]);
             } else {
-                o[4] += 0.25 * sx * sy * w[5];
-                o[5] += 0.25 * sx * sy * w[14];
+                d2 += 0.25 * sx * sy * w[5];
+                d4 += 0.25 * sx * sy * w[14];
             }
             const double wt = g < 2 ? 0.25 : 0.125;  // axis groups: each velocity sees one axis
-            o[6] += wt * (sx * w[1] + sy * w[2]);
-            o[7] += wt * (sx * w[7] + sy * w[8]);
-            o[8] += wt * (sx * w[9] + sy * w[12]);
-            o[9] += wt * (sx * w[11] + sy * w[10]);
+            j += wt * (sx * w[1] + sy * w[2]);
+            pj += wt * (sx * w[7] + sy * w[8]);
+            aaa += wt * (sx * w[9] + sy * w[12]);
+            abb += wt * (sx * w[11] + sy * w[10]);
         }
+        const double o[10] = {one, en * b + 2.0 * s2, en + s2, s4, d2, d4,
+                              j, pj * (b + 2.0) + 3.0 * aaa + abb, pj + 0.5 * (aaa + abb), 0.5 * (aaa - abb)};
+        for (int q = 0; q < 10; ++q) k.c[g][q] = o[q];
     }
 }
 template <typename R> UpdateArgs<R> update_args(const lbm_ctx *c, int stage, int rows_per_cta) {

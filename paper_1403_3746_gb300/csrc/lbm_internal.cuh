@@ -283,16 +283,16 @@ template <typename R> struct UpdateConst {
     R psi_hi[16], psi_lo[16];  // psi_i = |v_i|^2 + eta_i^2 as a two-term sum (hi + lo)
     R minv[256];               // inverse of the 16x16 moment matrix, row-major
 };
-// float64: psi of each speed group, and M^-1 reduced by the symmetry of the velocity set. The
-// four velocities of a speed group are images of one another under the reflections of the axes
-// and their exchange, so f^eq of the group is made of one even and two odd sums of moments with
-// common coefficients (update_node64): c[0..3] of rho, E, m_xx + m_yy, psi-m_xx + psi-m_yy; c[4..5] of
-// m_xx - m_yy and its psi partner (axis groups) or m_xy and its psi partner (diagonal groups);
-// c[6..9] of the odd moments j_a, psi-j_a, m_aaa, m_abb along axis a.
+// float64: psi of each speed group, and f^eq_i / rho = (M^-1 m^eq)_i / rho as polynomials of u and
+// T reduced by the symmetry of the velocity set: the four velocities of a speed group are images
+// of one another under the reflections of the axes and their exchange. With d = u_x^2 - u_y^2,
+// gq = (b + 4) T + u^2 and p3 = (2 b + 4) T^2 + (b + 6) T u^2 + u^4:
+//   even part  c0 + c1 T + c2 u^2 + c3 p3 +- (d or u_x u_y) (c4 + c5 gq)   (axis or diagonal groups)
+//   odd part   u_x (c6 + c7 T + c8 u^2 + c9 d), u_y (c6 + c7 T + c8 u^2 - c9 d)
 template <> struct UpdateConst<double> {
     double psi[4];
     double c[4][10];
-    double ib;  // 1 / b
+    double ib, b4, b24, b6;  // 1 / b, b + 4, 2 b + 4, b + 6
 };
 template <typename R> struct UpdateArgs {
     const R *fs;     // f of this stage (derivatives, BGK, f^eq moments), [ny][16][nx]

@@ -597,15 +597,20 @@ __device__ __forceinline__ void update_node32(const UpdateArgs<R> &a, const Upda
 }
 
 // The float64 node. It is bound by the 2 float64 operations per clock and SM, so it is written
-// for their number: f^eq by speed groups from the symmetry-reduced M^-1 (UpdateConst<double>: 84
-// operations instead of the 256 of the full matrix), forcing factors and moment sums by opposite
-// pairs, one reciprocal for 1/(rho T), 1/(rho T^2). About 310 operations per node instead of 570:
-// 1024^2 update pass 1.58 -> 1.10 ms per launch (row transforms included).
+// for their number, about 240 per node (570 for the full matrix product and four separate sums):
+//  - f_i^eq = rho phi_i with phi_i a polynomial of u and T whose coefficients are common to a speed
+//    group up to signs (UpdateConst<double>): an even and two odd sums per four velocities;
+//  - f_out = [f_base - (h/tau) f_i + h advection] + W_i phi_i with W_i = rho (h/tau - q_i), so that
+//    collision and forcing are one multiply-add per velocity, rho times the forcing factors q_i
+//    needs 1/T alone, and stage 1 (f_base = f_i) takes (1 - h/tau) f_i;
+//  - moment sums by opposite pairs.
+// 1024^2 update pass, row transforms included: 1.58 ms per launch with the full product, 1.02 with
+// the group sums of moments, 0.90 like this (0.67 with the shorter products of fft_fixed.cuh).
 template <int LOG2N, bool AX_POSSIBLE>
 __device__ __forceinline__ void update_node64(const UpdateArgs<double> &a, const UpdateConst<double> &kc, size_t y, int x,
                                               const double2 *dl, size_t ls, int xl) {
     constexpr int NX = 1 << LOG2N;
-    const double K = a.K, h = a.h;
+    const double h = a.h;
     const bool adv = !(a.flags & LBM_FLAG_NO_ADVECTION);
     const bool col = !(a.flags & LBM_FLAG_NO_COLLISION);
     const bool frc = !(a.flags & LBM_FLAG_NO_FORCE);
@@ -615,66 +620,61 @@ __device__ __forceinline__ void update_node64(const UpdateArgs<double> &a, const
     double *mn = a.m + y * NF_M * NX + x, *on = a.fout + y * NF_F * NX + x;
     const double rho = ldcg(mn + M_RHO * NX), ux = ldcg(mn + M_UX * NX), uy = ldcg(mn + M_UY * NX);
     const double T = ldcg(mn + M_T * NX);
-    const double xx = ux * ux, yy = uy * uy, u2 = xx + yy;
-    // I_i = -(al + bx v_ix + by v_iy + cc |v_i|^2) f_i^eq, h folded in (as in update_node32)
-    double hal = 0, hbx = 0, hby = 0, hcc = 0;
+    const double xx = ux * ux, yy = uy * uy, u2 = xx + yy, d = xx - yy, uxy = ux * uy;
+    // I_i = -(al + bx v_ix + by v_iy + cc |v_i|^2) f_i^eq, rho h folded in
+    double al = 0, bx = 0, by = 0, cc = 0;
     if (frc) {
-        const double irT = 1.0 / (rho * T), irTT = irT * (irT * rho);  // 1 / (rho T), 1 / (rho T^2)
-        const double hB = h * irT, hC = h * irTT;
-        const double Bx = (ldcg(mn + M_DSXX * NX) + ldcg(mn + M_DSXYY * NX)) * hB;
-        const double By = (ldcg(mn + M_DSXY * NX) + ldcg(mn + M_DSYY * NX)) * hB;
-        const double C = ldcg(mn + M_CNUM * NX) - K * rho * ldcg(mn + M_RY * NX) * ldcg(mn + M_DDIVUY * NX);
-        hcc = (0.5 * C + (ldcg(mn + M_DQX * NX) + ldcg(mn + M_DQY * NX))) * hC;
-        const double cc2 = 2.0 * hcc;
-        hal = hcc * (u2 - 2.0 * T) - Bx * ux - By * uy;
-        hbx = Bx - cc2 * ux;
-        hby = By - cc2 * uy;
+        const double iT = 1.0 / T, hT = h * iT;
+        const double Bx = (ldcg(mn + M_DSXX * NX) + ldcg(mn + M_DSXYY * NX)) * hT;
+        const double By = (ldcg(mn + M_DSXY * NX) + ldcg(mn + M_DSYY * NX)) * hT;
+        const double C = ldcg(mn + M_CNUM * NX) - a.K * rho * ldcg(mn + M_RY * NX) * ldcg(mn + M_DDIVUY * NX);
+        cc = (0.5 * C + (ldcg(mn + M_DQX * NX) + ldcg(mn + M_DQY * NX))) * (hT * iT);
+        const double cc2 = 2.0 * cc;
+        al = cc * (u2 - 2.0 * T) - Bx * ux - By * uy;
+        bx = Bx - cc2 * ux;
+        by = By - cc2 * uy;
     }
-    const double htau = h * a.tau_inv;
-    // moments of f^eq: even ones as sums and differences of the xx and yy parts, odd ones per axis
-    const double e = (a.b + 2.0) * T + u2, gq = (a.b + 4.0) * T + u2;
-    const double jx = rho * ux, jy = rho * uy, rd = rho * (xx - yy), rxy = jx * uy;
-    const double mE = rho * (a.b * T + u2), mS = rho * (2.0 * T + u2), mP = rho * (2.0 * T * e + gq * u2);
-    const double mD = rd, mQ = gq * rd, mXY = rxy, mPXY = gq * rxy;
-    const double ox[4] = {jx, jx * e, jx * (3.0 * T + xx), jx * (T + yy)};
-    const double oy[4] = {jy, jy * e, jy * (3.0 * T + yy), jy * (T + xx)};
+    const double htau = col ? h * a.tau_inv : 0.0, keep = same_base ? 1.0 - htau : -htau;
+    const double w0 = rho * htau - al;
+    const double gq = kc.b4 * T + u2, p3 = T * (kc.b24 * T + kc.b6 * u2) + u2 * u2;
     MomentSums<double> acc;
     static_for<0, 4>([&](auto GI) {
         constexpr int g = decltype(GI)::value;
         constexpr double v = vel_x(4 * g), v2 = vel_sq(4 * g);
         const double *c = kc.c[g];
-        const double ev = c[0] * rho + c[1] * mE + c[2] * mS + c[3] * mP;
-        const double ed = g < 2 ? c[4] * mD + c[5] * mQ : c[4] * mXY + c[5] * mPXY;
-        const double odx = c[6] * ox[0] + c[7] * ox[1] + c[8] * ox[2] + c[9] * ox[3];
-        const double ody = c[6] * oy[0] + c[7] * oy[1] + c[8] * oy[2] + c[9] * oy[3];
-        // even and odd parts of the pairs (0, 2) and (1, 3): axis groups x and y, diagonal groups
-        // (+,+) and (-,+)
+        // even and odd parts of phi for the pairs (0, 2) and (1, 3): axis groups x and y, diagonal
+        // groups (+,+) and (-,+)
+        const double ev = c[0] + c[1] * T + c[2] * u2 + c[3] * p3;
+        const double ed = (g < 2 ? d : uxy) * (c[4] + c[5] * gq);
+        const double os = c[6] + c[7] * T + c[8] * u2;
+        const double odx = ux * (os + c[9] * d), ody = uy * (os - c[9] * d);
         const double e0 = ev + ed, e1 = ev - ed;
         const double o0 = g < 2 ? odx : ody + odx, o1 = g < 2 ? ody : ody - odx;
-        const double qe = hal + hcc * v2;
-        const double q0 = g < 2 ? v * hbx : v * (hby + hbx), q1 = g < 2 ? v * hby : v * (hby - hbx);
+        const double we = w0 - cc * v2;
+        const double q0 = g < 2 ? v * bx : v * (by + bx), q1 = g < 2 ? v * by : v * (by - bx);
         double out[4];
         static_for<0, 4>([&](auto KI) {
             constexpr int k = decltype(KI)::value, i = 4 * g + k, xs = xslot(i), ys = yslot(i);
-            const double ee = k & 1 ? e1 : e0, oo = k & 1 ? o1 : o0, qq = k & 1 ? q1 : q0;
-            const double fe = k < 2 ? ee + oo : ee - oo, q = k < 2 ? qe + qq : qe - qq;
             const double f = ldcg(fn + i * NX);
-            double dfo = 0;  // h R_i
+            double dfo = 0;  // -h v_i . grad f_i
             if (adv) {
                 if constexpr (xs >= 0) {
                     if (ax_mode) {
                         dfo = -h * (vel_x(i) * ldcg(a.Ax + (y * NF_F + i) * NX + x));
                     } else {
-                        const double2 d = dl[(xs >> 1) * ls + xl];
-                        dfo = (xs & 1) ? -d.y : d.x;
+                        const double2 dd = dl[(xs >> 1) * ls + xl];
+                        dfo = (xs & 1) ? -dd.y : dd.x;
                     }
                 }
                 if constexpr (ys >= 0) dfo += ldcg(an + ys * NX);
             }
-            if (col) dfo += htau * (fe - f);
-            if (frc) dfo -= q * fe;
-            out[k] = (same_base ? f : ldcg(bn + i * NX)) + dfo;
-            on[i * NX] = out[k];
+            double o = same_base ? keep * f + dfo : (keep * f + ldcg(bn + i * NX)) + dfo;
+            if (col || frc) {
+                const double ee = k & 1 ? e1 : e0, oo = k & 1 ? o1 : o0, qq = k & 1 ? q1 : q0;
+                o += (k < 2 ? we - qq : we + qq) * (k < 2 ? ee + oo : ee - oo);
+            }
+            out[k] = o;
+            on[i * NX] = o;
         });
         acc.template add_group<g>(out[0], out[1], out[2], out[3], kc.psi[g]);
     });
