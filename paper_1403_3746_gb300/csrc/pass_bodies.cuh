@@ -125,159 +125,164 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
         if constexpr (RHO64) prefetch_l2(a.r64 + (size_t)(y0 + threadIdx.x) * NR64 * NX, NR64 * NX * sizeof(double));
     }
 
-    // round 1: derivatives of the moments along x
-    CT v[E];
-    for (int kind = my_kind; kind <= (SERIAL ? 1 : my_kind); ++kind) {
-        if (!active) {  // the barriers of the line groups (A then B in turn when SERIAL, else B)
-            for (int k = 0; k < (SERIAL ? 2 : 1); ++k) {
-                F::template idle_forward<reg::SyncCta>();
+    // Line rounds: 0: first derivatives of the moments along x; 1: d_xx rho from line A's spectrum
+    // (B waits); then the nodes; 2: d_x of (Q_x, S_xx) on line A and of (S_xy, div u) on line B. In
+    // float64 a loop, so that the long fixed-point transforms exist once in the code: unrolled (two
+    // forward, three inverse) the pass's warps waited for instructions more than for anything else
+    // (5.6 of 13 cycles per instruction; 1024^2 426 -> 255 us per launch, 64^2 51 -> 33, together with
+    // the shorter products). The float32 transforms fit the instruction cache unrolled and are
+    // faster so (1024^2 31.2 against 32.8 us, 4096^2 545 against 611).
+    typename F::Scale sc0;
+    auto line_round = [&](int it) {
+        if (!active) {  // the barriers of the line groups
+            for (int k = 0; k < (SERIAL && it != 1 ? 2 : 1); ++k) {
+                if (it != 1) F::template idle_forward<reg::SyncCta>();
+                F::template idle_inverse<reg::SyncCta>();
+                if (it != 2) reg::cta_barrier();
+            }
+            return;
+        }
+        for (int kind = my_kind; kind <= (SERIAL && it != 1 ? 1 : my_kind); ++kind) {
+            if (it == 1 && kind == 1) {
                 F::template idle_inverse<reg::SyncCta>();
                 reg::cta_barrier();
-                if (!SERIAL || k == 0) F::template idle_inverse<reg::SyncCta>();
-                reg::cta_barrier();
+                continue;
             }
-            break;
-        }
-        CT *O1 = buf1(kind);
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int x = t + G * e;
-            v[e] = kind == 0 ? reg::mk<R>(__ldcg(mrow + M_RHO * NX + x), __ldcg(mrow + M_T * NX + x))
-                             : reg::mk<R>(__ldcg(mrow + M_UX * NX + x), __ldcg(mrow + M_UY * NX + x));
-        }
-        const typename F::Scale sc0 = F::template forward<reg::SyncCta>(v, O1, t, a.ax, 1);
-        if (kind == 0) F::storeF(v, O2, t);  // keep the spectrum of A for d_xx rho (thread-private slots)
-        typename F::Scale sc = sc0;
-        F::multiply(v, t, 1, R(1), a.ax, sc);
-        F::template inverse<reg::SyncCta>(v, O1, t, a.ax, sc, 1);
-        reg::cta_barrier();
-#pragma unroll
-        for (int e = 0; e < E; ++e) O1[t + G * e] = v[e];
-        if (kind == 0) {
-            F::loadF(v, O2, t);
-            sc = sc0;
-            F::multiply(v, t, 2, R(1), a.ax, sc);
-            F::template inverse<reg::SyncCta>(v, O2, t, a.ax, sc, 1);
-        } else if (!SERIAL) {
-            F::template idle_inverse<reg::SyncCta>();
-        }
-        reg::cta_barrier();
-        if (kind == 0) {
-#pragma unroll
-            for (int e = 0; e < E; ++e) O2[t + G * e] = v[e];
-        }
-    }
-    __syncthreads();
-
-    using D = std::conditional_t<RHO64, double, R>;  // type of the rho-dependent terms
-    const D K = RHO64 ? (D)a.K64 : (D)a.K, H = RHO64 ? (D)a.H64 : (D)a.H, q = RHO64 ? (D)a.q64 : (D)a.q,
-            zeta = RHO64 ? (D)a.zeta64 : (D)a.zeta;
-    static_assert(!DIAG || (sizeof(R) == 4 && !RHO64 && !SERIAL), "fused diagnostics: float32 pass only");
-    FPair dS[DIAG ? 5 : 1];
-    for (int idx = threadIdx.x; idx < nodes; idx += blockDim.x) {
-        const int rr = idx / NX, x = idx % NX;
-        R *mn = a.m + (size_t)(y0 + rr) * NF_M * NX + x;  // this node: field k at mn[k * NX]
-        CT *A1 = lines + (size_t)rr * 3 * SM, *A2 = A1 + SM, *B1 = A1 + 2 * SM;
-        const D Tx = A1[x].y;
-        const D dux_dx = B1[x].x, duy_dx = B1[x].y;
-        const D T = __ldcg(mn + M_T * NX);
-        const D dux_dy = __ldcg(mn + M_UXY * NX), duy_dy = __ldcg(mn + M_UYY * NX);
-        const D Ty = __ldcg(mn + M_TY * NX);
-        D rho, rx, rxx, ry, ryy;
-        if constexpr (RHO64) {
-            const double *rn = a.r64 + (size_t)(y0 + rr) * NR64 * NX + x;
-            rho = __ldcg(rn + R64_RHO * NX);
-            rx = __ldcg(rn + R64_RX * NX);
-            rxx = __ldcg(rn + R64_RXX * NX);
-            ry = __ldcg(rn + R64_RY * NX);
-            ryy = __ldcg(rn + R64_RYY * NX);
-            mn[M_RY * NX] = (R)ry;  // read by the update pass's C term
-        } else {
-            rho = __ldcg(mn + M_RHO * NX);
-            rx = A1[x].x;
-            rxx = A2[x].x;
-            ry = __ldcg(mn + M_RY * NX);
-            ryy = __ldcg(mn + M_RYY * NX);
-        }
-
-        if constexpr (DIAG)
-            diag_accumulate(dS, (float)rho, __ldcg(mn + M_UX * NX), __ldcg(mn + M_UY * NX), (float)T, (float)rx,
-                            (float)ry, a.diag_hK);
-
-        const D lap = rxx + ryy;
-        const D divu = dux_dx + duy_dy;
-        // van der Waals EOS (Sec. 2.2)
-        const D rT = rho * T;
-        D iT2, Pw;
-        if constexpr (sizeof(D) == 8) {  // one division for both quotients
-            const D d3 = D(3) - rho, T2 = T * T, r = D(1) / (d3 * T2);
-            iT2 = d3 * r;
-            Pw = D(3) * rT * (T2 * r) - D(1.125) * rho * rho;
-        } else {
-            iT2 = quot(D(1), T * T);
-            Pw = quot(D(3) * rT, D(3) - rho) - D(1.125) * rho * rho;
-        }
-        // Lambda with M = K + H T and grad(M/T) = -K grad T / T^2
-        const D Mc = K + H * T;
-        const D gx = -K * Tx * iT2, gy = -K * Ty * iT2;
-        const D grr = rx * rx + ry * ry;
-        const D iso = Mc * (rho * lap + D(0.5) * grr) + rT * (rx * gx + ry * gy);
-        const D Lxx = Mc * rx * rx - iso, Lxy = Mc * rx * ry, Lyy = Mc * ry * ry - iso;
-        const D Pn = Pw - rT - zeta * divu;
-        const D Sxx = Pn + Lxx, Sxy = Lxy, Syy = Pn + Lyy;
-        const D qrT = q * rT;
-        const D Qx = qrT * Tx, Qy = qrT * Ty;
-        // numerator of C without -K rho (d_x rho d_x(div u) + d_y rho d_y(div u)): the x term is
-        // added after round 2 below, the y term by the update pass (after the flux pass)
-        const D L_gradu = Lxx * dux_dx + Lxy * (duy_dx + dux_dy) + Lyy * duy_dy;
-        const D r_gradu_r = rx * (dux_dx * rx + duy_dx * ry) + ry * (dux_dy * rx + duy_dy * ry);
-        mn[M_CNUM * NX] = (R)((Pw - rT) * divu + L_gradu - zeta * divu * divu + D(1.125) * rho * rho * divu +
-                              K * (-D(0.5) * grr * divu - r_gradu_r));
-        if constexpr (SERIAL) mn[M_DSXY * NX] = (R)(K * rho * rx);
-        else A2[x].y = (R)(K * rho * rx);  // this thread read A2[x].x above
-        mn[M_QY * NX] = (R)Qy;
-        mn[M_SXY * NX] = (R)Sxy;
-        mn[M_SYY * NX] = (R)Syy;
-        mn[M_DIVU * NX] = (R)divu;
-        A1[x] = reg::mk<R>((R)Qx, (R)Sxx);  // round-2 lines, same node and thread as the reads above
-        B1[x] = reg::mk<R>((R)Sxy, (R)divu);
-    }
-    if constexpr (DIAG) {
-        __shared__ float dwarp[32][5][2];
-        diag_warp_reduce(dS, dwarp);
-        __syncthreads();
-        diag_block_write(dwarp, a.diag_partial + (size_t)blk * 5);
-    }
-    __syncthreads();
-
-    // round 2: d_x of (Q_x, S_xx) on line A and of (S_xy, div u) on line B
-    for (int kind = my_kind; kind <= (SERIAL ? 1 : my_kind); ++kind) {
-        if (!active) {
-            for (int k = 0; k < (SERIAL ? 2 : 1); ++k) {
-                F::template idle_forward<reg::SyncCta>();
-                F::template idle_inverse<reg::SyncCta>();
-            }
-            break;
-        }
-        CT *O1 = buf1(kind);
-#pragma unroll
-        for (int e = 0; e < E; ++e) v[e] = O1[t + G * e];
-        typename F::Scale sc = F::template forward<reg::SyncCta>(v, O1, t, a.ax, 1);
-        F::multiply(v, t, 1, R(1), a.ax, sc);
-        F::template inverse<reg::SyncCta>(v, O1, t, a.ax, sc, 1);
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int x = t + G * e;
-            if (kind == 0) {
-                mrow[M_DQX * NX + x] = v[e].x;
-                mrow[M_DSXX * NX + x] = v[e].y;
+            CT *O = it == 1 ? O2 : buf1(kind);
+            CT v[E];
+            typename F::Scale sc;
+            if (it == 1) {
+                F::loadF(v, O2, t);
+                sc = sc0;
             } else {
-                // - K rho d_x rho d_x(div u); the partial value was written by this CTA's node loop
-                const R k = SERIAL ? mrow[M_DSXY * NX + x] : O2[x].y;
-                mrow[M_DSXY * NX + x] = v[e].x;
-                mrow[M_CNUM * NX + x] -= k * v[e].y;
+                if (it == 0) {
+                    const R *pa = mrow + (kind == 0 ? M_RHO : M_UX) * NX, *pb = mrow + (kind == 0 ? M_T : M_UY) * NX;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) v[e] = reg::mk<R>(__ldcg(pa + t + G * e), __ldcg(pb + t + G * e));
+                } else {
+#pragma unroll
+                    for (int e = 0; e < E; ++e) v[e] = O[t + G * e];
+                }
+                sc = F::template forward<reg::SyncCta>(v, O, t, a.ax, 1);
+                if (!RHO64 && it == 0 && kind == 0) {  // keep the spectrum of A for d_xx rho (thread-private slots)
+                    F::storeF(v, O2, t);
+                    sc0 = sc;
+                }
+            }
+            F::multiply(v, t, it == 1 ? 2 : 1, R(1), a.ax, sc);
+            F::template inverse<reg::SyncCta>(v, O, t, a.ax, sc, 1);
+            if (it < 2) {
+                reg::cta_barrier();
+#pragma unroll
+                for (int e = 0; e < E; ++e) O[t + G * e] = v[e];
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int x = t + G * e;
+                    if (kind == 0) {
+                        mrow[M_DQX * NX + x] = v[e].x;
+                        mrow[M_DSXX * NX + x] = v[e].y;
+                    } else {
+                        // - K rho d_x rho d_x(div u); the partial value was written by this CTA's node loop
+                        const R k = SERIAL ? mrow[M_DSXY * NX + x] : O2[x].y;
+                        mrow[M_DSXY * NX + x] = v[e].x;
+                        mrow[M_CNUM * NX + x] -= k * v[e].y;
+                    }
+                }
             }
         }
+    };
+
+    auto nodes_loop = [&]() {
+        using D = std::conditional_t<RHO64, double, R>;  // type of the rho-dependent terms
+        const D K = RHO64 ? (D)a.K64 : (D)a.K, H = RHO64 ? (D)a.H64 : (D)a.H, q = RHO64 ? (D)a.q64 : (D)a.q,
+                zeta = RHO64 ? (D)a.zeta64 : (D)a.zeta;
+        static_assert(!DIAG || (sizeof(R) == 4 && !RHO64 && !SERIAL), "fused diagnostics: float32 pass only");
+        FPair dS[DIAG ? 5 : 1];
+        for (int idx = threadIdx.x; idx < nodes; idx += blockDim.x) {
+            const int rr = idx / NX, x = idx % NX;
+            R *mn = a.m + (size_t)(y0 + rr) * NF_M * NX + x;  // this node: field k at mn[k * NX]
+            CT *A1 = lines + (size_t)rr * 3 * SM, *A2 = A1 + SM, *B1 = A1 + 2 * SM;
+            const D Tx = A1[x].y;
+            const D dux_dx = B1[x].x, duy_dx = B1[x].y;
+            const D T = __ldcg(mn + M_T * NX);
+            const D dux_dy = __ldcg(mn + M_UXY * NX), duy_dy = __ldcg(mn + M_UYY * NX);
+            const D Ty = __ldcg(mn + M_TY * NX);
+            D rho, rx, rxx, ry, ryy;
+            if constexpr (RHO64) {
+                const double *rn = a.r64 + (size_t)(y0 + rr) * NR64 * NX + x;
+                rho = __ldcg(rn + R64_RHO * NX);
+                rx = __ldcg(rn + R64_RX * NX);
+                rxx = __ldcg(rn + R64_RXX * NX);
+                ry = __ldcg(rn + R64_RY * NX);
+                ryy = __ldcg(rn + R64_RYY * NX);
+                mn[M_RY * NX] = (R)ry;  // read by the update pass's C term
+            } else {
+                rho = __ldcg(mn + M_RHO * NX);
+                rx = A1[x].x;
+                rxx = A2[x].x;
+                ry = __ldcg(mn + M_RY * NX);
+                ryy = __ldcg(mn + M_RYY * NX);
+            }
+
+            if constexpr (DIAG)
+                diag_accumulate(dS, (float)rho, __ldcg(mn + M_UX * NX), __ldcg(mn + M_UY * NX), (float)T, (float)rx,
+                                (float)ry, a.diag_hK);
+
+            const D lap = rxx + ryy;
+            const D divu = dux_dx + duy_dy;
+            // van der Waals EOS (Sec. 2.2)
+            const D rT = rho * T;
+            D iT2, Pw;
+            if constexpr (sizeof(D) == 8) {  // one division for both quotients
+                const D d3 = D(3) - rho, T2 = T * T, r = D(1) / (d3 * T2);
+                iT2 = d3 * r;
+                Pw = D(3) * rT * (T2 * r) - D(1.125) * rho * rho;
+            } else {
+                iT2 = quot(D(1), T * T);
+                Pw = quot(D(3) * rT, D(3) - rho) - D(1.125) * rho * rho;
+            }
+            // Lambda with M = K + H T and grad(M/T) = -K grad T / T^2
+            const D Mc = K + H * T;
+            const D gx = -K * Tx * iT2, gy = -K * Ty * iT2;
+            const D grr = rx * rx + ry * ry;
+            const D iso = Mc * (rho * lap + D(0.5) * grr) + rT * (rx * gx + ry * gy);
+            const D Lxx = Mc * rx * rx - iso, Lxy = Mc * rx * ry, Lyy = Mc * ry * ry - iso;
+            const D Pn = Pw - rT - zeta * divu;
+            const D Sxx = Pn + Lxx, Sxy = Lxy, Syy = Pn + Lyy;
+            const D qrT = q * rT;
+            const D Qx = qrT * Tx, Qy = qrT * Ty;
+            // numerator of C without -K rho (d_x rho d_x(div u) + d_y rho d_y(div u)): the x term is
+            // added after round 2 below, the y term by the update pass (after the flux pass)
+            const D L_gradu = Lxx * dux_dx + Lxy * (duy_dx + dux_dy) + Lyy * duy_dy;
+            const D r_gradu_r = rx * (dux_dx * rx + duy_dx * ry) + ry * (dux_dy * rx + duy_dy * ry);
+            mn[M_CNUM * NX] = (R)((Pw - rT) * divu + L_gradu - zeta * divu * divu + D(1.125) * rho * rho * divu +
+                                  K * (-D(0.5) * grr * divu - r_gradu_r));
+            if constexpr (SERIAL) mn[M_DSXY * NX] = (R)(K * rho * rx);
+            else A2[x].y = (R)(K * rho * rx);  // this thread read A2[x].x above
+            mn[M_QY * NX] = (R)Qy;
+            mn[M_SXY * NX] = (R)Sxy;
+            mn[M_SYY * NX] = (R)Syy;
+            mn[M_DIVU * NX] = (R)divu;
+            A1[x] = reg::mk<R>((R)Qx, (R)Sxx);  // round-2 lines, same node and thread as the reads above
+            B1[x] = reg::mk<R>((R)Sxy, (R)divu);
+        }
+        if constexpr (DIAG) {
+            __shared__ float dwarp[32][5][2];
+            diag_warp_reduce(dS, dwarp);
+            __syncthreads();
+            diag_block_write(dwarp, a.diag_partial + (size_t)blk * 5);
+        }
+    };
+
+#pragma unroll(sizeof(R) == 8 ? 1 : 3)
+    for (int it = 0; it < 3; it += RHO64 ? 2 : 1) {  // (d_xx rho from the density chain)
+        if (it == 2) {
+            __syncthreads();
+            nodes_loop();
+            __syncthreads();
+        }
+        line_round(it);
     }
 }
 
