@@ -151,6 +151,8 @@ struct lbm_ctx {
     // one captured step (both stages) for lbm_step when timing is off
     cudaStream_t cap = nullptr;
     cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph_many = nullptr;  // kManySteps steps
+    long long graph_steps = 0;             // steps launched as graphs
 
     // per-launch timing
     bool timing = false;
@@ -175,6 +177,8 @@ struct lbm_batch_ctx {
     std::vector<cudaEvent_t> join;
     cudaEvent_t fork = nullptr;
     cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph_many = nullptr;        // kManySteps steps: the groups run them independently
+    long long graph_steps = 0;                   // steps launched as graphs
     std::vector<long long> steps;                // per instance, since its lbm_batch_init
     // persistent form (kernels_batch.cu): one launch per step over all instances
     int form = LBM_BATCH_GRAPH;
@@ -560,14 +564,22 @@ int capture_into(lbm_ctx *c, cudaStream_t s) {
     return rc;
 }
 
+// Steps per launch of c->graph_many (c's own steps, or a batch's), and the steps a handle takes one by
+// one before that graph is built: a graph's launch costs 4.1 us against 0.7 to 1.2 us per kernel
+// within one, and building one of 64 kernels a fraction of a millisecond, which a handle of few
+// steps does not pay. @MANY@
+constexpr int kManySteps = 8, kManyAfter = 32;
+
 // One step's launches as a CUDA graph: c->graph, or for a fused diagnostics request in slot
 // `slot` (>= 0) c->graph_diag[slot], whose first macro pass also writes the diagnostics partial
 // values into fpart[slot].
-int build_step_graph(lbm_ctx *c, int slot = -1) {
+// count > 1: that many steps, into c->graph_many.
+int build_step_graph(lbm_ctx *c, int slot = -1, int count = 1) {
     if (!c->cap) CU_TRY(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
     CU_TRY(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed));
     c->fuse_capture = slot;
-    const int rc = capture_into(c, c->cap);
+    int rc = LBM_OK;
+    for (int k = 0; k < count && rc == LBM_OK; ++k) rc = capture_into(c, c->cap);
     c->fuse_capture = -1;
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(c->cap, &g);
@@ -576,7 +588,8 @@ int build_step_graph(lbm_ctx *c, int slot = -1) {
         return rc;
     }
     CU_TRY(e);
-    const cudaError_t ei = cudaGraphInstantiate(slot >= 0 ? &c->graph_diag[slot] : &c->graph, g, 0);
+    const cudaError_t ei =
+        cudaGraphInstantiate(slot >= 0 ? &c->graph_diag[slot] : count > 1 ? &c->graph_many : &c->graph, g, 0);
     cudaGraphDestroy(g);
     CU_TRY(ei);
     return LBM_OK;
@@ -586,6 +599,8 @@ int build_step_graph(lbm_ctx *c, int slot = -1) {
 void drop_graphs(lbm_ctx *c) {
     if (c->graph) cudaGraphExecDestroy(c->graph);
     c->graph = nullptr;
+    if (c->graph_many) cudaGraphExecDestroy(c->graph_many);
+    c->graph_many = nullptr;
     for (cudaGraphExec_t &g : c->graph_diag) {
         if (g) cudaGraphExecDestroy(g);
         g = nullptr;
@@ -826,6 +841,7 @@ void free_ctx(lbm_ctx *c) {
     else cudaDeviceSynchronize();
     if (c->dstream) cudaStreamSynchronize(c->dstream);
     if (c->graph) cudaGraphExecDestroy(c->graph);
+    if (c->graph_many) cudaGraphExecDestroy(c->graph_many);
     for (int k = 0; k < 2; ++k) {
         if (c->graph_diag[k]) cudaGraphExecDestroy(c->graph_diag[k]);
         if (c->fpart[k]) cudaFree(c->fpart[k]);
@@ -1465,13 +1481,22 @@ int lbm_step(lbm_handle c, int n) {
         }
         return LBM_OK;
     }
-    if (!c->graph) {
+    // a handle that keeps stepping runs kManySteps steps per graph
+    while (n >= kManySteps && c->graph_steps >= kManyAfter) {
+        if (!c->graph_many && build_step_graph(c, -1, kManySteps)) break;  // one by one then
+        CU_TRY(cudaGraphLaunch(c->graph_many, c->stream));
+        c->steps += kManySteps;
+        c->graph_steps += kManySteps;
+        n -= kManySteps;
+    }
+    if (n > 0 && !c->graph) {
         int rc = build_step_graph(c);
         if (rc) return rc;
     }
-    for (int s = 0; s < n; ++s) {
+    for (; n > 0; --n) {
         CU_TRY(cudaGraphLaunch(c->graph, c->stream));
         ++c->steps;
+        ++c->graph_steps;
     }
     return LBM_OK;
 }
@@ -1903,6 +1928,7 @@ void lbm_batch_destroy(lbm_batch b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     else cudaDeviceSynchronize();
     if (b->graph) cudaGraphExecDestroy(b->graph);
+    if (b->graph_many) cudaGraphExecDestroy(b->graph_many);
     if (b->pgraph) cudaGraphExecDestroy(b->pgraph);
     if (b->bctrl) cudaFree(b->bctrl);
     for (cudaStream_t s : b->branch) cudaStreamDestroy(s);
@@ -2006,6 +2032,10 @@ int lbm_batch_autotune(lbm_batch b) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
     }
+    if (b->graph_many) {
+        cudaGraphExecDestroy(b->graph_many);
+        b->graph_many = nullptr;
+    }
     if (b->form == LBM_BATCH_PERSISTENT) return autotune_persistent(b);
     return LBM_OK;
 }
@@ -2026,7 +2056,7 @@ int lbm_batch_init(lbm_batch b, int k, const double *rho, const double *ux, cons
 
 // One graph per step: the groups' launches are parallel branches forked from and joined back
 // into the capture stream.
-static int build_batch_graph(lbm_batch b) {
+static int build_batch_graph(lbm_batch b, int count) {
     const size_t G = b->groups.size();
     if (!b->cap) CU_TRY(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
     if (!b->fork) CU_TRY(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
@@ -2047,7 +2077,7 @@ static int build_batch_graph(lbm_batch b) {
     cudaError_t e = cudaEventRecord(b->fork, b->cap);
     for (size_t g = 0; g < G && rc == LBM_OK && e == cudaSuccess; ++g) {
         e = cudaStreamWaitEvent(b->branch[g], b->fork, 0);
-        if (e == cudaSuccess) rc = capture_into(b->groups[g], b->branch[g]);
+        for (int k = 0; k < count && rc == LBM_OK && e == cudaSuccess; ++k) rc = capture_into(b->groups[g], b->branch[g]);
         if (rc == LBM_OK && e == cudaSuccess) e = cudaEventRecord(b->join[g], b->branch[g]);
         if (rc == LBM_OK && e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->join[g], 0);
     }
@@ -2059,7 +2089,7 @@ static int build_batch_graph(lbm_batch b) {
         return fail(LBM_ERR_CUDA, "batch graph capture: %s",
                     cudaGetErrorString(e != cudaSuccess ? e : ee));
     }
-    const cudaError_t ei = cudaGraphInstantiate(&b->graph, graph, 0);
+    const cudaError_t ei = cudaGraphInstantiate(count > 1 ? &b->graph_many : &b->graph, graph, 0);
     cudaGraphDestroy(graph);
     CU_TRY(ei);
     return LBM_OK;
@@ -2246,11 +2276,20 @@ int lbm_batch_step(lbm_batch b, int n) {
         for (long long &s : b->steps) s += n;
         return LBM_OK;
     }
-    if (!b->graph) {
-        int rc = build_batch_graph(b);
+    int left = n;
+    for (; left >= kManySteps && b->graph_steps >= kManyAfter; left -= kManySteps) {
+        if (!b->graph_many && build_batch_graph(b, kManySteps)) break;  // one by one then
+        CU_TRY(cudaGraphLaunch(b->graph_many, b->stream));
+        b->graph_steps += kManySteps;
+    }
+    if (left > 0 && !b->graph) {
+        int rc = build_batch_graph(b, 1);
         if (rc) return rc;
     }
-    for (int s = 0; s < n; ++s) CU_TRY(cudaGraphLaunch(b->graph, b->stream));
+    for (; left > 0; --left) {
+        CU_TRY(cudaGraphLaunch(b->graph, b->stream));
+        ++b->graph_steps;
+    }
     for (long long &s : b->steps) s += n;
     return LBM_OK;
 }
