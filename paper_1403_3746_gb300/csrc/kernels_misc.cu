@@ -85,18 +85,67 @@ __global__ void moments_kernel(const __grid_constant__ MomArgs a) {
     }
 }
 
-// LBM_MIXED_RHO64: rho of every node as the float64 sum of its 16 stored float32 values (exact:
-// the values span far fewer than the 29 bits a float64 has beyond a float32's significand).
-__global__ void rho64_kernel(const float *f, double *r64, int nx, int ny) {
+// LBM_MIXED_RHO64: rho of every node as the sum of its 16 stored float32 values, exact to 2^-56 and
+// then rounded once to float64. The sum runs in 64-bit integers of unit 2^-56 (|f| < 4), because the
+// 31 conversions and additions of the float64 form take 16 clocks of an SM's float64 unit per node
+// (with the one-launch row pass below, 1024^2: 188 -> 120 us per stage for the whole chain); nodes with a larger, infinite or NaN value take that form.
+__global__ void __launch_bounds__(256) rho64_kernel(const float *f, double *r64, int nx, int ny) {
     const long long n = (long long)nx * ny;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n;
          g += (long long)gridDim.x * blockDim.x) {
         const long long y = g / nx, x = g - y * nx;
         const float *fn = f + y * NF_F * nx + x;
-        double s = 0.0;
+        unsigned bits[16], top = 0;
+        long long sum = 0;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) s += (double)__ldcg(fn + i * nx);
+        for (int i = 0; i < 16; ++i) bits[i] = __float_as_uint(__ldcg(fn + i * nx));
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const unsigned a = bits[i] & 0x7fffffffu;
+            top = max(top, a);
+            const int sh = (int)(a >> 23) - 94;  // unit 2^-56
+            const unsigned m = (a & 0x7fffffu) | 0x800000u;
+            const unsigned long long v = sh >= 0 ? (unsigned long long)m << (sh & 63) : (unsigned long long)(m >> min(-sh, 31));
+            sum += (int)bits[i] < 0 ? -(long long)v : (long long)v;
+        }
+        double s;
+        if (top < 0x40800000u) {  // every |f| < 4
+            s = __longlong_as_double((long long)fixed::to_double(sum, -56));
+        } else {
+            s = 0.0;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) s += (double)__uint_as_float(bits[i]);
+        }
         r64[(y * NR64 + R64_RHO) * nx + x] = s;
+    }
+}
+
+// LBM_MIXED_RHO64: d_x rho and d_xx rho of the float64 density in one launch. A complex line packs
+// rows 2 j and 2 j + 1; its spectrum waits in a second buffer for the second derivative: three
+// transforms per two rows, where two launches of the general row derivative took eight.
+template <int LOG2N>
+__global__ void __launch_bounds__(256, 2) rho64_row_kernel(double *r64, const __grid_constant__ Axis<double> ax) {
+    using F = reg::Line<double, LOG2N, false>;
+    constexpr int NX = F::N, G = F::G, E = F::E, SM = F::STRIDE;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int slot = threadIdx.x / G, t = threadIdx.x % G;
+    double2 *buf = reinterpret_cast<double2 *>(smem_raw) + (size_t)slot * 2 * SM, *spec = buf + SM;
+    double *row = r64 + (size_t)(blockIdx.x * (blockDim.x / G) + slot) * 2 * NR64 * NX, *row1 = row + NR64 * NX;
+    double2 v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        v[e] = make_double2(__ldcg(row + R64_RHO * NX + t + G * e), __ldcg(row1 + R64_RHO * NX + t + G * e));
+    const typename F::Scale sc0 = F::template forward<reg::SyncCta>(v, buf, t, ax, 1);
+    F::storeF(v, spec, t);  // thread-private slots
+#pragma unroll 1
+    for (int order = 1; order <= 2; ++order) {
+        typename F::Scale sc = sc0;
+        if (order == 2) F::loadF(v, spec, t);
+        F::multiply(v, t, order, 1.0, ax, sc);
+        F::template inverse<reg::SyncCta>(v, buf, t, ax, sc, 1);
+        const int o = (order == 1 ? R64_RX : R64_RXX) * NX + t;
+#pragma unroll
+        for (int e = 0; e < E; ++e) row[o + G * e] = v[e].x, row1[o + G * e] = v[e].y;
     }
 }
 
@@ -242,6 +291,27 @@ static inline int grid_for(long long n) {
 cudaError_t launch_rho64(const float *f, double *r64, int nx, int ny, cudaStream_t s) {
     rho64_kernel<<<grid_for((long long)nx * ny), 256, 0, s>>>(f, r64, nx, ny);
     return cudaGetLastError();
+}
+
+template <int LOG2N> static cudaError_t launch_rho64_rows_n(double *r64, const Axis<double> &ax, int ny, cudaStream_t s) {
+    using F = reg::Line<double, LOG2N, false>;
+    // about 128 threads per CTA: two CTAs' line buffers fit an SM at 1024 points
+    int lines = F::G < 128 ? 128 / F::G : 1;
+    while ((ny / 2) % lines) lines >>= 1;
+    const size_t smem = (size_t)lines * 2 * F::STRIDE * sizeof(double2);
+    cudaError_t e = allow_smem(rho64_row_kernel<LOG2N>);
+    if (e != cudaSuccess) return e;
+    rho64_row_kernel<LOG2N><<<ny / (2 * lines), lines * F::G, smem, s>>>(r64, ax);
+    return cudaGetLastError();
+}
+cudaError_t launch_rho64_rows(double *r64, const Axis<double> &ax, int ny, cudaStream_t s) {
+    switch (ax.log2n) {
+#define LBM_CASE(L2) \
+    case L2: return launch_rho64_rows_n<L2>(r64, ax, ny, s);
+        LBM_FOR_LOG2N(LBM_CASE)
+#undef LBM_CASE
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // Validity of initial fields (0 < rho < 3, T > 0 and finite, u finite): the lowest index of a

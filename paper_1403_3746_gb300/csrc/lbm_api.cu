@@ -315,7 +315,7 @@ template <typename R> MacroArgs<R> macro_args(const lbm_ctx *c, int rows_per_cta
 }
 
 // LBM_MIXED_RHO64: rho of the stage's f as a float64 sum, then its derivatives by float64
-// transforms: d_y rho, d_yy rho (one column launch) and d_x rho, d_xx rho (two row launches).
+// transforms: d_y rho, d_yy rho (one column launch) and d_x rho, d_xx rho (one row launch).
 int run_rho64_chain(lbm_ctx *c, const float *fs) {
     const int nx = c->nx, rows = c->nb * c->ny, ld = NR64 * nx;
     double *r = c->r64;
@@ -326,19 +326,7 @@ int run_rho64_chain(lbm_ctx *c, const float *fs) {
     ca.jobs[0] = ColJob<double>{F(R64_RHO), F(R64_RY), ld, ld, 1, 1.0};
     ca.jobs[1] = ColJob<double>{F(R64_RHO), F(R64_RYY), ld, ld, 2, 1.0};
     CU_TRY(launch_col<double>(ca, 2, c->geo64.col_smem, c->stream));
-    for (int order = 1; order <= 2; ++order) {
-        RowDerivArgs<double> ra{};
-        ra.in[0] = F(R64_RHO);
-        ra.out[0] = F(order == 1 ? R64_RX : R64_RXX);
-        ra.ld = ld;
-        ra.nin = 1;
-        ra.nx = nx;
-        ra.ny = rows;
-        ra.rows = c->geo64.rows_rowd;
-        ra.order = order;
-        ra.ax = axis<double>(c, true);
-        CU_TRY(launch_row_deriv<double>(ra, c->geo64.rowd_smem, c->stream));
-    }
+    CU_TRY(launch_rho64_rows(r, axis<double>(c, true), rows, c->stream));
     return LBM_OK;
 }
 
