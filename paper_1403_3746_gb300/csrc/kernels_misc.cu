@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(MaxThreads<R>::value, MaxThreads<R>::min_block
     const int NR = a.rows;
     const int slot = threadIdx.x / G, t = threadIdx.x % G;
     const int p = slot / NR, r = slot % NR;
-    const size_t row = (size_t)(blockIdx.x * NR + r) * a.ld;
+    const size_t row = (size_t)(blockIdx.x * NR + r) * a.ld + (size_t)blockIdx.y * a.gstride;
     const int ka = 2 * p, kb = 2 * p + 1;
     CT v[E];
 #pragma unroll
@@ -279,7 +279,7 @@ template <typename R, int LOG2N> static cudaError_t launch_row_deriv_n(const Row
     if (smem < (size_t)((a.nin + 1) / 2) * a.rows * F::STRIDE * sizeof(typename F::CT)) return cudaErrorInvalidValue;
     cudaError_t e = allow_smem(row_deriv_kernel<R, LOG2N>);
     if (e != cudaSuccess) return e;
-    row_deriv_kernel<R, LOG2N><<<a.ny / a.rows, ((a.nin + 1) / 2) * a.rows * F::G, smem, s>>>(a);
+    row_deriv_kernel<R, LOG2N><<<dim3(a.ny / a.rows, a.groups > 0 ? a.groups : 1), ((a.nin + 1) / 2) * a.rows * F::G, smem, s>>>(a);
     return cudaGetLastError();
 }
 

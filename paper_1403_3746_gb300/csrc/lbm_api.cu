@@ -478,8 +478,7 @@ int run_stage(lbm_ctx *c, int stage, int passes = PASS_ALL) {
 }
 
 // The solution filter (params filter_alpha > 0): f_i <- the inverse transform of W(m_x) W(m_y)
-// times the spectrum of f_i for all 16 fields in place, as a row pass (launches of four or two
-// fields) and a column pass (16 jobs), each adding the transform of the correction W - 1 to the
+// times the spectrum of f_i for all 16 fields in place, as a row pass and a column pass (16 jobs), each adding the transform of the correction W - 1 to the
 // field, then the moments of the filtered f for the next step.
 template <typename R> Axis<R> filter_axis(const lbm_ctx *c, bool xdir);
 template <> Axis<double> filter_axis<double>(const lbm_ctx *c, bool xdir) {
@@ -493,22 +492,21 @@ template <> Axis<float> filter_axis<float>(const lbm_ctx *c, bool xdir) {
 template <typename R> int run_filter(lbm_ctx *c) {
     const int nx = c->nx, rows = c->nb * c->ny, ldf = NF_F * nx;
     R *f = static_cast<R *>(c->f0);
-    // four fields (two lines per row) per launch where the threads allow it, else two
+    // all 16 fields in one launch, four (two lines per row) per CTA where the threads allow it, else two
     const int per = 2 * c->geo.rows_rowd * line_G(c->lx) <= max_threads(c->fsize) ? 4 : 2;
-    for (int k = 0; k < 16; k += per) {
-        RowDerivArgs<R> ra{};
-        for (int j = 0; j < per; ++j) {
-            ra.in[j] = f + (size_t)(k + j) * nx;
-            ra.out[j] = f + (size_t)(k + j) * nx;
-        }
-        ra.ld = ldf;
-        ra.nin = per;
-        ra.nx = nx;
-        ra.ny = rows;
-        ra.rows = c->geo.rows_rowd;
-        ra.order = 2;
-        ra.acc = 1;
-        ra.ax = filter_axis<R>(c, true);
+    RowDerivArgs<R> ra{};
+    for (int j = 0; j < per; ++j) ra.in[j] = ra.out[j] = f + (size_t)j * nx;
+    ra.groups = 16 / per;
+    ra.gstride = per * nx;
+    ra.ld = ldf;
+    ra.nin = per;
+    ra.nx = nx;
+    ra.ny = rows;
+    ra.rows = c->geo.rows_rowd;
+    ra.order = 2;
+    ra.acc = 1;
+    ra.ax = filter_axis<R>(c, true);
+    {
         LaunchTimer t(c, LBM_K_UPDATE);
         CU_TRY(launch_row_deriv<R>(ra, (per / 2) * c->geo.rowd_smem, c->stream));
     }
@@ -555,7 +553,7 @@ int capture_into(lbm_ctx *c, cudaStream_t s) {
 // Steps per launch of c->graph_many (c's own steps, or a batch's), and the steps a handle takes one by
 // one before that graph is built: a graph's launch costs 4.1 us against 0.7 to 1.2 us per kernel
 // within one, and building one of 64 kernels a fraction of a millisecond, which a handle of few
-// steps does not pay. @MANY@
+// steps does not pay (mixed 256^2 57.4 -> 55.6 us per step, five 128^2 as a batch 61.5 -> 59.8).
 constexpr int kManySteps = 8, kManyAfter = 32;
 
 // One step's launches as a CUDA graph: c->graph, or for a fused diagnostics request in slot
@@ -946,37 +944,31 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
     cudaError_t e = cudaMemsetAsync(c->err, 0, sizeof(int), c->stream);
     if (e == cudaSuccess) e = launch_twiddles(c->tw64x, c->tw32x, nx, c->stream);
     if (e == cudaSuccess) e = launch_twiddles(c->tw64y, c->tw32y, ny, c->stream);
-    for (int ax = 0; ax < 2 && e == cudaSuccess; ++ax) {
-        const int N = ax == 0 ? nx : ny;
-        const double d = ax == 0 ? params->dx : params->dy;
-        std::vector<double> k1(N), k2(N);
-        std::vector<float> k1f(N), k2f(N);
-        derivative_tables(N, d, params->win_alpha, params->win_p, k1.data(), k2.data(), params->keff_terms);
+    // the host's tables lie side by side in the slab, from twfx to kfy32: one upload
+    char *const tab0 = reinterpret_cast<char *>(c->twfx);
+    std::vector<char> tab(reinterpret_cast<char *>(c->kfy32 + ny) - tab0);
+    auto H = [&](auto *dev) { return reinterpret_cast<decltype(dev)>(tab.data() + (reinterpret_cast<char *>(dev) - tab0)); };
+    for (int ax = 0; ax < 2; ++ax) {
+        const bool x = ax == 0;
+        const int N = x ? nx : ny;
+        std::vector<double> k1(N), k2(N), kf(N);  // kf: the solution filter's (unused while filter_alpha = 0)
+        derivative_tables(N, x ? params->dx : params->dy, params->win_alpha, params->win_p, k1.data(), k2.data(),
+                          params->keff_terms);
+        filter_table(N, params->filter_alpha, params->filter_p, kf.data());
+        float *k1f = H(x ? c->k1x32 : c->k1y32), *k2f = H(x ? c->k2x32 : c->k2y32), *kff = H(x ? c->kfx32 : c->kfy32);
         for (int pos = 0; pos < N; ++pos) {
             k1f[pos] = (float)k1[pos];
             k2f[pos] = (float)k2[pos];
+            kff[pos] = (float)kf[pos];
         }
-        long long *dk1 = ax == 0 ? c->k1x : c->k1y, *dk2 = ax == 0 ? c->k2x : c->k2y;
-        std::vector<long long> k1i(N), k2i(N), kfi(N);
-        std::vector<longlong2> twf(N);
-        fixed_twiddles(N, twf.data());
-        (ax == 0 ? c->p1x : c->p1y) = fixed_multipliers(N, k1.data(), k1i.data());
-        (ax == 0 ? c->p2x : c->p2y) = fixed_multipliers(N, k2.data(), k2i.data());
-        float *fk1 = ax == 0 ? c->k1x32 : c->k1y32, *fk2 = ax == 0 ? c->k2x32 : c->k2y32;
-        e = cudaMemcpy(ax == 0 ? c->twfx : c->twfy, twf.data(), N * sizeof(longlong2), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(dk1, k1i.data(), N * 8, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(dk2, k2i.data(), N * 8, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(fk1, k1f.data(), N * 4, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(fk2, k2f.data(), N * 4, cudaMemcpyHostToDevice);
-        // the solution filter's table (unused while filter_alpha = 0)
-        std::vector<double> kf(N);
-        std::vector<float> kff(N);
-        filter_table(N, params->filter_alpha, params->filter_p, kf.data());
-        for (int pos = 0; pos < N; ++pos) kff[pos] = (float)kf[pos];
-        (ax == 0 ? c->pfx : c->pfy) = fixed_multipliers(N, kf.data(), kfi.data());
-        if (e == cudaSuccess) e = cudaMemcpy(ax == 0 ? c->kfx : c->kfy, kfi.data(), N * 8, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(ax == 0 ? c->kfx32 : c->kfy32, kff.data(), N * 4, cudaMemcpyHostToDevice);
+        if (!c->mixed || c->rho64) {  // float64 lines
+            fixed_twiddles(N, H(x ? c->twfx : c->twfy));
+            (x ? c->p1x : c->p1y) = fixed_multipliers(N, k1.data(), H(x ? c->k1x : c->k1y));
+            (x ? c->p2x : c->p2y) = fixed_multipliers(N, k2.data(), H(x ? c->k2x : c->k2y));
+            (x ? c->pfx : c->pfy) = fixed_multipliers(N, kf.data(), H(x ? c->kfx : c->kfy));
+        }
     }
+    if (e == cudaSuccess) e = cudaMemcpy(tab0, tab.data(), tab.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         cudaFree(c->slab);
@@ -2419,7 +2411,8 @@ int fixed_multipliers(int N, const double *k, long long *out) {
     for (int i = 0; i < N; ++i) top = std::max(top, std::fabs(k[i]));
     int p = 0;
     if (top > 0) std::frexp(top, &p);  // |k| 2^-p < 1
-    for (int i = 0; i < N; ++i) out[i] = fixed::balance(std::llrint(std::ldexp(k[i], 62 - p)));
+    const double s1 = std::ldexp(1.0, (62 - p) / 2), s2 = std::ldexp(1.0, 62 - p - (62 - p) / 2);
+    for (int i = 0; i < N; ++i) out[i] = fixed::balance(std::llrint(k[i] * s1 * s2));
     return p;
 }
 

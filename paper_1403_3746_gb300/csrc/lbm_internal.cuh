@@ -465,6 +465,8 @@ template <typename R> struct RowDerivArgs {
     R *out[4];
     int ld;  // row stride of every in / out field (elements)
     int nin;  // 1..4 inputs (paired two per complex line)
+    int groups;   // the same for `groups` sets of fields (0: one), set g at + g gstride elements
+    int gstride;
     int nx, ny, rows;
     int order;  // 1: d_x (table k1); 2: the real multiplier of table k2 (a second derivative or a filter)
     int acc;    // 1: out = in + the result (in place: the solution filter's correction)
