@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(256, 2) rho64_row_kernel(double *r64, const __
 // float32 pipe (GB300's float64 rate is 1/64 of float32); the block's sums become float64 once.
 template <typename R>
 __global__ void __launch_bounds__(256) diag_kernel(const __grid_constant__ DiagArgs a) {
+    if (a.err && blockIdx.x == 0 && threadIdx.x == 0) a.partial[gridDim.x * 5] = (double)*a.err;
     const R *prho = static_cast<const R *>(a.rho), *pux = static_cast<const R *>(a.ux);
     const R *puy = static_cast<const R *>(a.uy), *pT = static_cast<const R *>(a.T);
     const R *prx = static_cast<const R *>(a.rx), *pry = static_cast<const R *>(a.ry);
@@ -223,15 +224,18 @@ __global__ void twiddle_kernel(double2 *tw64, float2 *tw32, int n) {
     }
 }
 
-// out[y][x] = src[y ld + x] as float64
-template <typename R>
-__global__ void field_out_kernel(const R *src, int ld, double *out, int nx, int ny) {
-    const long long n = (long long)nx * ny;
+// out[j][y][x] = src[j][y ld + x] as float64 for up to four fields (blockIdx.y; a null output is
+// skipped), and the device error word as a float64 behind the last one where the caller wants it with
+// the same copy.
+template <typename R> __global__ void fields_out_kernel(const __grid_constant__ FieldsOutArgs a) {
+    double *out = a.out[blockIdx.y];
+    if (a.err_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *a.err_out = (double)*a.err;
+    if (!out) return;
+    const R *src = static_cast<const R *>(a.src[blockIdx.y]);
+    const long long n = (long long)a.nx * a.ny;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n;
-         g += (long long)gridDim.x * blockDim.x) {
-        const long long y = g / nx, x = g - y * nx;
-        out[g] = (double)src[y * ld + x];
-    }
+         g += (long long)gridDim.x * blockDim.x)
+        out[g] = (double)src[(g >> a.lx) * a.ld + (g & (a.nx - 1))];
 }
 
 // Generic spectral x-derivative (or, order 2, the real multiplier of table k2: a second
@@ -348,9 +352,8 @@ cudaError_t launch_twiddles(double2 *tw64, float2 *tw32, int n, cudaStream_t s) 
     twiddle_kernel<<<(n + 255) / 256, 256, 0, s>>>(tw64, tw32, n);
     return cudaGetLastError();
 }
-template <typename R>
-cudaError_t launch_field_out(const R *src, int ld, double *out, int nx, int ny, cudaStream_t s) {
-    field_out_kernel<R><<<grid_for((long long)nx * ny), 256, 0, s>>>(src, ld, out, nx, ny);
+template <typename R> cudaError_t launch_fields_out(const FieldsOutArgs &a, cudaStream_t s) {
+    fields_out_kernel<R><<<dim3(grid_for((long long)a.nx * a.ny), 4), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 template <typename R>
@@ -368,8 +371,8 @@ template cudaError_t launch_init<double>(const InitArgs &, cudaStream_t);
 template cudaError_t launch_init<float>(const InitArgs &, cudaStream_t);
 template cudaError_t launch_moments<double>(const MomArgs &, cudaStream_t);
 template cudaError_t launch_moments<float>(const MomArgs &, cudaStream_t);
-template cudaError_t launch_field_out<double>(const double *, int, double *, int, int, cudaStream_t);
-template cudaError_t launch_field_out<float>(const float *, int, double *, int, int, cudaStream_t);
+template cudaError_t launch_fields_out<double>(const FieldsOutArgs &, cudaStream_t);
+template cudaError_t launch_fields_out<float>(const FieldsOutArgs &, cudaStream_t);
 template cudaError_t launch_row_deriv<double>(const RowDerivArgs<double> &, size_t, cudaStream_t);
 template cudaError_t launch_row_deriv<float>(const RowDerivArgs<float> &, size_t, cudaStream_t);
 template cudaError_t launch_diag<double>(const DiagArgs &, int, cudaStream_t);

@@ -911,7 +911,7 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
     parts.push_back({&c->m, (size_t)NF_M * plane_f});
     if (c->geo.upd_ax) parts.push_back({&c->Ax, 16 * plane_f});
     if (c->rho64) parts.push_back({reinterpret_cast<void **>(&c->r64), (size_t)NR64 * c->n * nb * sizeof(double)});
-    parts.push_back({reinterpret_cast<void **>(&c->partial), (size_t)c->diag_blocks * 5 * 8});
+    parts.push_back({reinterpret_cast<void **>(&c->partial), ((size_t)c->diag_blocks * 5 + 1) * 8});
     parts.push_back({reinterpret_cast<void **>(&c->err), sizeof(int)});
     parts.push_back({reinterpret_cast<void **>(&c->bad), sizeof(unsigned long long)});
     parts.push_back({reinterpret_cast<void **>(&c->tw64x), (size_t)nx * 16});
@@ -992,17 +992,23 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
 
 // After a synchronisation of the context's stream: the error word of the bounded device
 // waits. A set word is reported once (and cleared) as LBM_ERR_TIMEOUT.
-int check_device_error(lbm_ctx *c) {
-    int v = 0;
-    CU_TRY(cudaMemcpyAsync(&v, c->err, sizeof v, cudaMemcpyDeviceToHost, c->stream));
-    CU_TRY(cudaStreamSynchronize(c->stream));
-    if (v == 0) return LBM_OK;
+// (device_error: for a word v != 0 that was read already)
+int device_error(lbm_ctx *c, int v) {
     CU_TRY(cudaMemsetAsync(c->err, 0, sizeof v, c->stream));
     CU_TRY(cudaStreamSynchronize(c->stream));
     return fail(LBM_ERR_TIMEOUT, "a bounded device-side wait gave up (error word %d): the steps since the last "
                 "check did not complete and the state is not valid",
                 v);
 }
+int check_device_error(lbm_ctx *c) {
+    int v = 0;
+    CU_TRY(cudaMemcpyAsync(&v, c->err, sizeof v, cudaMemcpyDeviceToHost, c->stream));
+    CU_TRY(cudaStreamSynchronize(c->stream));
+    return v == 0 ? LBM_OK : device_error(c, v);
+}
+// float64 values up to which a read-out goes through one host buffer (a copy in memory costs less than
+// three more copies from the device)
+constexpr size_t kSmallRead = 1 << 13;
 
 // f_i := f_i^eq(rho, u, T) for instance k from device arrays [ny][nx]
 int init_instance(lbm_ctx *c, int k, const double *rho, const double *ux, const double *uy, const double *T) {
@@ -1042,34 +1048,54 @@ int init_instance_host(lbm_ctx *c, int k, const double *rho, const double *ux, c
     return init_instance(c, k, st, st + c->n, st + 2 * c->n, st + 3 * c->n);
 }
 
-// rho, u_x, u_y, T (macro fields 0..3) of instance k as dense float64 [ny][nx] device arrays
-int moments_to_device(lbm_ctx *c, int k, double *const out[4]) {
-    const int ld = NF_M * c->nx;
+// rho, u_x, u_y, T (macro fields 0..3) of instance k as dense float64 [ny][nx] device arrays in one
+// launch; err_out: also the error word
+int moments_to_device(lbm_ctx *c, int k, double *const out[4], double *err_out = nullptr) {
+    FieldsOutArgs a{};
+    a.ld = NF_M * c->nx;
+    a.nx = c->nx;
+    a.ny = c->ny;
+    a.lx = c->lx;
+    a.err = c->err;
+    a.err_out = err_out;
     for (int j = 0; j < 4; ++j) {
-        if (!out[j]) continue;
-        const size_t off = c->row0(k) * ld + (size_t)j * c->nx;
-        if (c->mixed)
-            CU_TRY(launch_field_out<float>(static_cast<const float *>(c->m) + off, ld, out[j], c->nx, c->ny,
-                                           c->stream));
-        else
-            CU_TRY(launch_field_out<double>(static_cast<const double *>(c->m) + off, ld, out[j], c->nx, c->ny,
-                                            c->stream));
+        a.src[j] = static_cast<const char *>(c->m) + (c->row0(k) * a.ld + (size_t)j * c->nx) * c->fsize;
+        a.out[j] = out[j];
     }
+    CU_TRY(c->mixed ? launch_fields_out<float>(a, c->stream) : launch_fields_out<double>(a, c->stream));
     return LBM_OK;
 }
 
+// Host read-out by as few copies and waits as the buffers allow (five copies and two waits cost a small
+// grid much of its read: 128^2, pinned arrays, 83 -> 56 us): the fields are gathered in the
+// half-step buffer with the error word behind them, and come back as one copy into the caller's
+// array where the four fields lie one after another in it, through a host buffer where they are
+// small, as one copy per field otherwise.
 int moments_host(lbm_ctx *c, int k, double *rho, double *ux, double *uy, double *T) {
-    // gather through the half-step buffer (free outside a step), 4 x n doubles <= its size
+    // 4 x n + 1 doubles <= the size of the half-step buffer (free outside a step, 16 values per node)
     double *st = static_cast<double *>(c->f1);
-    double *const dev[4] = {rho ? st : nullptr, ux ? st + c->n : nullptr, uy ? st + 2 * c->n : nullptr,
-                            T ? st + 3 * c->n : nullptr};
-    int rc = moments_to_device(c, k, dev);
-    if (rc) return rc;
+    const size_t n = (size_t)c->n;
     double *const host[4] = {rho, ux, uy, T};
-    for (int j = 0; j < 4; ++j)
-        if (host[j]) CU_TRY(cudaMemcpyAsync(host[j], dev[j], (size_t)c->n * 8, cudaMemcpyDeviceToHost, c->stream));
-    CU_TRY(cudaStreamSynchronize(c->stream));
-    return check_device_error(c);
+    double *const dev[4] = {rho ? st : nullptr, ux ? st + n : nullptr, uy ? st + 2 * n : nullptr, T ? st + 3 * n : nullptr};
+    double err = 0.0;
+    int rc = moments_to_device(c, k, dev, st + 4 * n);
+    if (rc) return rc;
+    if (4 * n <= kSmallRead) {
+        std::vector<double> buf(4 * n + 1);
+        CU_TRY(cudaMemcpyAsync(buf.data(), st, buf.size() * 8, cudaMemcpyDeviceToHost, c->stream));
+        CU_TRY(cudaStreamSynchronize(c->stream));
+        for (int j = 0; j < 4; ++j)
+            if (host[j]) std::memcpy(host[j], buf.data() + j * n, n * 8);
+        err = buf[4 * n];
+    } else {
+        const bool together = rho && ux == rho + n && uy == ux + n && T == uy + n;
+        if (together) CU_TRY(cudaMemcpyAsync(rho, st, 4 * n * 8, cudaMemcpyDeviceToHost, c->stream));
+        for (int j = 0; j < 4 && !together; ++j)
+            if (host[j]) CU_TRY(cudaMemcpyAsync(host[j], dev[j], n * 8, cudaMemcpyDeviceToHost, c->stream));
+        CU_TRY(cudaMemcpyAsync(&err, st + 4 * n, 8, cudaMemcpyDeviceToHost, c->stream));
+        CU_TRY(cudaStreamSynchronize(c->stream));
+    }
+    return err != 0.0 ? device_error(c, (int)err) : LBM_OK;
 }
 
 // the API's [16][ny][nx] float64 layout <-> the device block [ny][16][nx] of instance k
@@ -1273,6 +1299,7 @@ template <typename R> int diag_launch(lbm_ctx *c, int k) {
     da.ry = m + (size_t)M_QY * nx;
     da.ld = ldm;
     da.partial = c->partial;
+    da.err = c->err;
     da.nx = c->nx;
     da.ny = c->ny;
     da.K = c->p.K;
@@ -1284,10 +1311,10 @@ template <typename R> int diag_launch(lbm_ctx *c, int k) {
 int diagnostics_instance(lbm_ctx *c, int k, long long steps, double out[6]) {
     int rc = c->mixed ? diag_launch<float>(c, k) : diag_launch<double>(c, k);
     if (rc) return rc;
-    std::vector<double> part((size_t)c->diag_blocks * 5);
+    std::vector<double> part((size_t)c->diag_blocks * 5 + 1);  // the error word behind the partial values
     CU_TRY(cudaMemcpyAsync(part.data(), c->partial, part.size() * 8, cudaMemcpyDeviceToHost, c->stream));
     CU_TRY(cudaStreamSynchronize(c->stream));
-    if ((rc = check_device_error(c))) return rc;
+    if (part.back() != 0.0) return device_error(c, (int)part.back());
     double s[4] = {0, 0, 0, 0}, mx = 0;
     for (int b = 0; b < c->diag_blocks; ++b) {
         for (int j = 0; j < 4; ++j) s[j] += part[b * 5 + j];

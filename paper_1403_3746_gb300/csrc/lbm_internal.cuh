@@ -455,7 +455,8 @@ __device__ __forceinline__ void diag_block_write(const float (*wpart)[5][2], dou
 struct DiagArgs {
     const void *rho, *ux, *uy, *T, *rx, *ry;
     int ld;
-    double *partial;  // [blocks][5]
+    double *partial;  // [blocks][5], then the device error word where err is given
+    const int *err;
     int nx, ny;
     double K, cell;
 };
@@ -513,9 +514,15 @@ template <typename R> cudaError_t launch_init(const InitArgs &a, cudaStream_t s)
 template <typename R> cudaError_t launch_moments(const MomArgs &a, cudaStream_t s);
 template <typename R> cudaError_t launch_diag(const DiagArgs &a, int blocks, cudaStream_t s);
 cudaError_t launch_twiddles(double2 *tw64, float2 *tw32, int n, cudaStream_t s);
-// strided copies between a field of a block (row y at src + y ld) and a dense float64 array [ny][nx]
-template <typename R>
-cudaError_t launch_field_out(const R *src, int ld, double *out, int nx, int ny, cudaStream_t s);
+// dense float64 copies [ny][nx] of up to four fields of a block (row y at src + y ld), and the error word
+struct FieldsOutArgs {
+    const void *src[4];
+    double *out[4];  // nullptr: skipped
+    int ld, nx, ny, lx;
+    const int *err;
+    double *err_out;  // nullptr: not wanted
+};
+template <typename R> cudaError_t launch_fields_out(const FieldsOutArgs &a, cudaStream_t s);
 
 template <typename R> cudaError_t launch_structure_factor(const SfArgs &a, cudaStream_t s);
 // signed DFT index held at each position of a forward line transform of length N (lbm_api.cu)
