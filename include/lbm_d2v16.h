@@ -261,8 +261,8 @@ int lbm_autotune(lbm_handle h, int geometry[4], double ms[4]);
  * DRAM streams while the resident CTAs transform. kinds[2]: CTAs per row of the update pass, 1,
  * 2 or 4 (a cluster of two or four splits each row's transforms and node loop; float32 rows of
  * 2048 or more for two, of 4096 for four, one row per cluster). Defaults: LBM_COL_TMA1 for both column passes of LBM_MIXED and
- * LBM_MIXED_RHO64 handles whose columns have 2048 or more points (where the shape allows it),
- * LBM_COL_DIRECT otherwise; 4 CTAs per update row for float32 rows of 4096, 1 otherwise.
+ * LBM_MIXED_RHO64 handles whose columns have 32 to 256 or 2048 or more points (where the shape allows
+ * it), LBM_COL_DIRECT otherwise; 4 CTAs per update row for float32 rows of 4096, 1 otherwise.
  * lbm_autotune chooses them together with the tile widths and rows
  * per CTA. lbm_set_pass_kinds returns LBM_ERR_ARG for a choice the current shapes cannot take
  * (TMA forms and lookahead: rows of fewer than 16 bytes or cluster-split widths; TMA forms:

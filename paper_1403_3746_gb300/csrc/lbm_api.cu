@@ -2479,10 +2479,13 @@ void pass_geometry(int nx, int ny, size_t esize, Geometry *g, int nb) {
     while (W > 2 && ((W / 2) * line_G(ly) > colt || col_smem(W, ly, esize) > 100 * 1024)) W >>= 1;
     g->colW = g->fluxW = W;
     g->col_smem = g->flux_smem = col_smem(W, ly, esize);
-    // float32 columns of 2048+ points: the TMA form with one staging buffer (measured against the
-    // direct form: 2048^2 step 1.80 -> 1.70 ms, 4096^2 8.44 -> 8.29 ms); elsewhere the direct form
+    // the TMA form with one staging buffer for float32 columns of 2048+ points (against the direct form:
+    // 2048^2 step 1.80 -> 1.70 ms, 4096^2 8.44 -> 8.29 ms) and for those of 32 to 256 points, whose passes
+    // are one latency after another: the tile arrives by one instruction (128^2 step 47.5 -> 40.3 us, 256^2
+    // 54.4 -> 47.2, five 128^2 58.3 -> 49.3, each with the rows rule below; 4096 x 256 433 -> 422);
+    // direct between (512^2 105.5 direct, 108.1 TMA; 1024^2 352 and 354)
     g->col_kind = g->flux_kind = LBM_COL_DIRECT;
-    if (esize == 4 && ly >= 11 && ((size_t)nx * esize) % 16 == 0) {
+    if (esize == 4 && (ly >= 11 || (ly >= 5 && ly <= 8)) && ((size_t)nx * esize) % 16 == 0) {
         const size_t sm = col_tma_smem(nx, ny, W, esize, 1);
         if (sm > 0 && sm <= kMaxCtaSmem) g->col_kind = g->flux_kind = LBM_COL_TMA1;
     }
@@ -2493,10 +2496,12 @@ void pass_geometry(int nx, int ny, size_t esize, Geometry *g, int nb) {
     if (r0 < 1) r0 = 1;
     if (r0 > ny) r0 = ny;
     // float64 nodes are bound by each SM's own float64 unit: fewer rows per CTA until there is a CTA
-    // for each of the 152 SMs (64^2: 8 rows -> 1, update pass 67 -> 35 us per launch; float32 passes of
-    // small grids are bound by latency and gained nothing)
-    while (esize == 8 && r0 > 1 && (long long)ny * nb / r0 < 152) r0 >>= 1;
+    // for each of the 152 SMs (64^2: 8 rows -> 1, update pass 67 -> 35 us per launch)
+    const long long rows = (long long)ny * nb;
+    while (esize == 8 && r0 > 1 && rows / r0 < 152) r0 >>= 1;
     int r = r0;
+    // float32 update pass of small grids: until two CTAs per SM (128^2 step 48.4 -> 46.3 us)
+    while (esize == 4 && r > 1 && rows / r < 304) r >>= 1;
     while (r > 1 && 6 * r * SM > 200 * 1024) r >>= 1;  // update: 6 line buffers per row
     g->rows_upd = r;
     g->upd_smem = 6 * (size_t)r * SM;
@@ -2516,6 +2521,13 @@ void pass_geometry(int nx, int ny, size_t esize, Geometry *g, int nb) {
     // macro: 2 lines per row with 3 buffers
     auto macro_bytes = [&](int rr) { return macro_smem(rr, lx, esize); };
     const int mact = macro_threads(esize, lx);
+    // float64 macro pass: the lines of up to 128 threads per CTA, so that its warps share the fetch of
+    // the transforms' code, while there are 128 CTAs (512^2 step 780 -> 724 us, 128 x 256 181 -> 177,
+    // 256 x 2048 1250 -> 1174)
+    if (esize == 8) {
+        r = 1;
+        while (2 * r <= ny && 4 * r * G <= 128 && rows / (2 * r) >= 128) r *= 2;
+    }
     while (r > 1 && (2 * r * G > mact || macro_bytes(r) > 200 * 1024)) r >>= 1;
     g->rows_macro = r;
     g->macro_smem = macro_bytes(r);
