@@ -1066,11 +1066,10 @@ int moments_to_device(lbm_ctx *c, int k, double *const out[4], double *err_out =
     return LBM_OK;
 }
 
-// Host read-out by as few copies and waits as the buffers allow (five copies and two waits cost a small
-// grid much of its read: 128^2, pinned arrays, 83 -> 56 us): the fields are gathered in the
-// half-step buffer with the error word behind them, and come back as one copy into the caller's
-// array where the four fields lie one after another in it, through a host buffer where they are
-// small, as one copy per field otherwise.
+// Host read-out by as few copies and waits as the buffers allow (four launches, five copies and two
+// waits made much of a small grid's read: 512 x 2 strips 2884 -> 2830 us per pass of 100 steps and a
+// read): the fields are gathered in the half-step buffer with the error word behind them, and come
+// back as one copy through a host buffer where they are small, as one copy per field otherwise.
 int moments_host(lbm_ctx *c, int k, double *rho, double *ux, double *uy, double *T) {
     // 4 x n + 1 doubles <= the size of the half-step buffer (free outside a step, 16 values per node)
     double *st = static_cast<double *>(c->f1);
@@ -1088,9 +1087,8 @@ int moments_host(lbm_ctx *c, int k, double *rho, double *ux, double *uy, double 
             if (host[j]) std::memcpy(host[j], buf.data() + j * n, n * 8);
         err = buf[4 * n];
     } else {
-        const bool together = rho && ux == rho + n && uy == ux + n && T == uy + n;
-        if (together) CU_TRY(cudaMemcpyAsync(rho, st, 4 * n * 8, cudaMemcpyDeviceToHost, c->stream));
-        for (int j = 0; j < 4 && !together; ++j)
+        // (never as one copy: arrays that follow one another in the address space may be pinned apart)
+        for (int j = 0; j < 4; ++j)
             if (host[j]) CU_TRY(cudaMemcpyAsync(host[j], dev[j], n * 8, cudaMemcpyDeviceToHost, c->stream));
         CU_TRY(cudaMemcpyAsync(&err, st + 4 * n, 8, cudaMemcpyDeviceToHost, c->stream));
         CU_TRY(cudaStreamSynchronize(c->stream));
