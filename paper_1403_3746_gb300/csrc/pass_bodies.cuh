@@ -64,6 +64,23 @@ template <typename T> __device__ __forceinline__ T ldcg(const T *p) { return __l
 // physical operands here) instead of the IEEE division sequence.
 __device__ __forceinline__ float quot(float a, float b) { return __fdividef(a, b); }
 
+// Conversions between float32 values and the type D of an expression. float64 <-> float32 in integer
+// arithmetic, the same bits as the conversion instructions, which take the float64 unit (2 per clock
+// and SM); values outside float32's normal range (zeros among them) take those.
+template <typename D> __device__ __forceinline__ D widen(D x) { return x; }
+template <typename D, typename R> __device__ __forceinline__ std::enable_if_t<(sizeof(D) > sizeof(R)), D> widen(R x) {
+    const unsigned b = __float_as_uint(x), a = b & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u) return (D)x;
+    return __hiloint2double((int)(((a >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(a << 29));
+}
+template <typename R> __device__ __forceinline__ R narrow(R x) { return x; }
+template <typename R, typename D> __device__ __forceinline__ std::enable_if_t<(sizeof(D) > sizeof(R)), R> narrow(D x) {
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x), a = h & 0x7fffffffu;
+    if (a - 0x38100000u >= 0x47e00000u - 0x38100000u) return (R)x;
+    const unsigned v = ((a - 0x38000000u) << 3) | (l >> 29), rem = l & 0x1fffffffu;
+    return __uint_as_float((v + (rem + (v & 1u) > 0x10000000u ? 1u : 0u)) | (h & 0x80000000u));  // to nearest, ties to even
+}
+
 // compile-time loop: f(std::integral_constant<int, I>) for I = B .. E-1
 template <int B, int E, class Fn> __device__ __forceinline__ void static_for(Fn &&f) {
     if constexpr (B < E) {
@@ -203,11 +220,11 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
             const int rr = idx / NX, x = idx % NX;
             R *mn = a.m + (size_t)(y0 + rr) * NF_M * NX + x;  // this node: field k at mn[k * NX]
             CT *A1 = lines + (size_t)rr * 3 * SM, *A2 = A1 + SM, *B1 = A1 + 2 * SM;
-            const D Tx = A1[x].y;
-            const D dux_dx = B1[x].x, duy_dx = B1[x].y;
-            const D T = __ldcg(mn + M_T * NX);
-            const D dux_dy = __ldcg(mn + M_UXY * NX), duy_dy = __ldcg(mn + M_UYY * NX);
-            const D Ty = __ldcg(mn + M_TY * NX);
+            const D Tx = widen<D>(A1[x].y);
+            const D dux_dx = widen<D>(B1[x].x), duy_dx = widen<D>(B1[x].y);
+            const D T = widen<D>(__ldcg(mn + M_T * NX));
+            const D dux_dy = widen<D>(__ldcg(mn + M_UXY * NX)), duy_dy = widen<D>(__ldcg(mn + M_UYY * NX));
+            const D Ty = widen<D>(__ldcg(mn + M_TY * NX));
             D rho, rx, rxx, ry, ryy;
             if constexpr (RHO64) {
                 const double *rn = a.r64 + (size_t)(y0 + rr) * NR64 * NX + x;
@@ -216,7 +233,7 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
                 rxx = __ldcg(rn + R64_RXX * NX);
                 ry = __ldcg(rn + R64_RY * NX);
                 ryy = __ldcg(rn + R64_RYY * NX);
-                mn[M_RY * NX] = (R)ry;  // read by the update pass's C term
+                mn[M_RY * NX] = narrow<R>(ry);  // read by the update pass's C term
             } else {
                 rho = __ldcg(mn + M_RHO * NX);
                 rx = A1[x].x;
@@ -268,15 +285,16 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
             }
             // numerator of C without -K rho (d_x rho d_x(div u) + d_y rho d_y(div u)): the x term is
             // added after round 2, the y term by the update pass (after the flux pass)
-            mn[M_CNUM * NX] = (R)cnum;
-            if constexpr (SERIAL) mn[M_DSXY * NX] = (R)(K * rho * rx);
-            else A2[x].y = (R)(K * rho * rx);  // this thread read A2[x].x above
-            mn[M_QY * NX] = (R)Qy;
-            mn[M_SXY * NX] = (R)Sxy;
-            mn[M_SYY * NX] = (R)Syy;
-            mn[M_DIVU * NX] = (R)divu;
-            A1[x] = reg::mk<R>((R)Qx, (R)Sxx);  // round-2 lines, same node and thread as the reads above
-            B1[x] = reg::mk<R>((R)Sxy, (R)divu);
+            mn[M_CNUM * NX] = narrow<R>(cnum);
+            if constexpr (SERIAL) mn[M_DSXY * NX] = narrow<R>(K * rho * rx);
+            else A2[x].y = narrow<R>(K * rho * rx);  // this thread read A2[x].x above
+            const R sxy = narrow<R>(Sxy), dv = narrow<R>(divu);
+            mn[M_QY * NX] = narrow<R>(Qy);
+            mn[M_SXY * NX] = sxy;
+            mn[M_SYY * NX] = narrow<R>(Syy);
+            mn[M_DIVU * NX] = dv;
+            A1[x] = reg::mk<R>(narrow<R>(Qx), narrow<R>(Sxx));  // round-2 lines, same node and thread as the reads above
+            B1[x] = reg::mk<R>(sxy, dv);
         }
         if constexpr (DIAG) {
             __shared__ float dwarp[32][5][2];
