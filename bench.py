@@ -42,9 +42,9 @@ KERNEL_NAMES = {"col": "col_deriv_kernel", "macro": "macro_row_kernel", "flux": 
                 "update": "update_row_kernel"}
 FP64_PEAK_TFLOPS = 1.25  # GB300 nominal dense FP64 (no tensor path for this work)
 # FP64 flops of one step of the FP64 path per node (DADD + DMUL + 2 DFMA thread instructions
-# of its four kernels, counted by ncu at 1024^2: 5.35 GFLOP per step; the count does not
-# depend on the launch shapes)
-FP64_FLOP_PER_NODE_STEP = 5.353e9 / (1024 * 1024)
+# of its four kernels, counted by ncu at 1024^2: 0.863 GFLOP per step, the node arithmetic; the
+# line transforms are 64-bit integer work; the count does not depend on the launch shapes)
+FP64_FLOP_PER_NODE_STEP = 0.863e9 / (1024 * 1024)
 
 
 def peaks():
@@ -59,8 +59,8 @@ def peaks():
 # the device code of the passes (kernels, FFT engine, shared layouts and launch limits); the
 # host orchestration (lbm_api.cu, lbm_noalloc.cu) is not part of it, and the launch shapes a
 # profile was taken with are checked separately
-DEVICE_SOURCES = ("fft_reg.cuh", "kernels_batch.cu", "kernels_col.cu", "kernels_misc.cu", "kernels_row.cu",
-                  "kernels_sf.cu", "lbm_internal.cuh", "pass_bodies.cuh", "tma.cuh")
+DEVICE_SOURCES = ("fft_fixed.cuh", "fft_line.cuh", "fft_reg.cuh", "kernels_batch.cu", "kernels_col.cu",
+                  "kernels_misc.cu", "kernels_row.cu", "kernels_sf.cu", "lbm_internal.cuh", "pass_bodies.cuh", "tma.cuh")
 
 
 def source_digest():
