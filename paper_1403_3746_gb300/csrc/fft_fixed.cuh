@@ -7,7 +7,7 @@
 // exponent per complex line (block floating point).
 //
 // Scaling of a line of N = 2^LOG2N points. Let 2^e bound the magnitude of the line's 2 N real
-// numbers (from their exponents). Point x enters as round(x 2^(B - e)), |Re|, |Im| < 2^B. Every
+// numbers (from their exponents). Point x enters as trunc(x 2^(B - e)), |Re|, |Im| < 2^B. Every
 // radix-16 pass that has outer twiddles ends (forward) or begins (inverse) with a factor 1/4,
 // which the high half of the product with a root scaled to 2^62 gives for free. B is the largest
 // value for which a sum of moduli cannot reach 2^63 anywhere in the forward passes: moduli start
@@ -18,14 +18,16 @@
 // every LOG2N <= 12. So no line can overflow, whatever its values.
 //
 // Rounding: each product is rounded to the nearest integer up to a quarter unit, inputs are
-// rounded once at 2^(e - B) (B = 54 .. 58), and before the inverse the spectrum is shifted up as
+// cut off once at 2^(e - B) (B = 54 .. 58), and before the inverse the spectrum is shifted up as
 // far as the sum of its magnitudes allows. Error of a derivative against __float128 sums, relative
 // to the float64 transform's, 8 .. 4096 points: 0.1 to 0.8 for lines with a mean, smooth, noisy or
 // step-like ones and for peaks a few points wide (1.06 for those at 4096), 1.8 to 2.8 for lines that
 // are zero but for one point (8e-16 of the result at most).
 //
-// Measured against the float64 transforms (1024^2, float64 step): column pass 1230 -> 524 us per
-// launch of 17 fields, flux pass 332 -> 160, step 8.31 -> 5.46 ms.
+// Measured against the float64 transforms (1024^2): column pass 1225 -> 240 us per launch of 17
+// fields, flux pass 330 -> 76; float64 step 8.31 -> 5.46 ms by the fixed-point lines alone, 2.32
+// with the node loops and launch shapes that followed. Both integer pipes are half busy (52 and
+// 55%) at 16 warps per SM.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -179,8 +181,9 @@ template <int LOG2N> __host__ __device__ __forceinline__ int line_bits(int c) {
     return b > base ? b : base;
 }
 
-// x 2^(B - e), truncated (the inputs' unit lies below what the passes round at), from the bits of the double x; e = emax - 1022 (emax: the largest exponent
-// field of the line, kMinExp <= emax <= 2046), top = emax + kMaxBits - B
+// x 2^(B - e), truncated (the inputs' unit lies below what the passes round at), from the bits of
+// the double x; e = emax - 1022 (emax: the largest exponent field of the line, kMinExp <= emax <=
+// 2046), top = emax + kMaxBits - B
 __host__ __device__ __forceinline__ long long from_double(unsigned long long x, int top) {
     const int hi = (int)(x >> 32);
     int d = top - (int)(((unsigned)hi >> 20) & 0x7ffu);

@@ -88,7 +88,8 @@ __global__ void moments_kernel(const __grid_constant__ MomArgs a) {
 // LBM_MIXED_RHO64: rho of every node as the sum of its 16 stored float32 values, exact to 2^-56 and
 // then rounded once to float64. The sum runs in 64-bit integers of unit 2^-56 (|f| < 4), because the
 // 31 conversions and additions of the float64 form take 16 clocks of an SM's float64 unit per node
-// (with the one-launch row pass below, 1024^2: 188 -> 120 us per stage for the whole chain); nodes with a larger, infinite or NaN value take that form.
+// (with the one-launch row pass below, 1024^2: 188 -> 120 us per stage for the whole chain); nodes
+// with a larger, infinite or NaN value take that form.
 __global__ void __launch_bounds__(256) rho64_kernel(const float *f, double *r64, int nx, int ny) {
     const long long n = (long long)nx * ny;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n;
