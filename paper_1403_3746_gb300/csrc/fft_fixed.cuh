@@ -7,27 +7,36 @@
 // exponent per complex line (block floating point).
 //
 // Scaling of a line of N = 2^LOG2N points. Let 2^e bound the magnitude of the line's 2 N real
-// numbers (from their exponents). Point x enters as trunc(x 2^(B - e)), |Re|, |Im| < 2^B. Every
-// radix-16 pass that has outer twiddles ends (forward) or begins (inverse) with a factor 1/4,
-// which the high half of the product with a root scaled to 2^62 gives for free. B is the largest
-// value for which a sum of moduli cannot reach 2^63 anywhere in the forward passes: moduli start
-// below 2^(B + 1/2), a radix-16 pass multiplies them by at most 16, so B = 62 - (largest growth).
-// The spectrum's 2-norm is at most N 2^(B + 1/2) / 4^T (T twiddled passes); the multiplier,
-// normalised to at most 1, is applied with another factor 1/4, and a sum of P of its points is at
-// most sqrt(P) times the 2-norm (Cauchy-Schwarz), which stays below 2^63 in every inverse pass for
-// every LOG2N <= 12. So no line can overflow, whatever its values.
+// numbers (from their exponents). Point x enters as trunc((x - c) 2^(B - e)). c is the line's mean,
+// taken out where that leaves more bits: every multiplier is zero at index 0, so a constant never
+// reaches the result. Every radix-16 pass that has outer twiddles ends (forward) or begins (inverse)
+// with a factor 1/4, which the high half of the product with a root scaled to 2^62 gives for free. B is
+// the largest value (line_bits) for which no sum can reach 2^63: a pass multiplies the largest
+// modulus by at most the points it has summed, and no sum of points passes the sum of all moduli.
 //
-// Rounding: each product is rounded to the nearest integer up to a quarter unit, inputs are
-// cut off once at 2^(e - B) (B = 54 .. 58), and before the inverse the spectrum is shifted up as
-// far as the sum of its magnitudes allows. Error of a derivative against __float128 sums, relative
-// to the float64 transform's, 8 .. 4096 points: 0.1 to 0.8 for lines with a mean, smooth, noisy or
-// step-like ones and for peaks a few points wide (1.06 for those at 4096), 1.8 to 2.8 for lines that
-// are zero but for one point (8e-16 of the result at most).
+// The spectrum is shifted up before it meets the multiplier, as far as its largest entry with a
+// non-zero multiplier allows, and the products again, until their summed magnitudes fill 2^63: the
+// mean and the low indices, whose multipliers are small, would otherwise leave the rest few bits.
+// Where the sum is larger than that without a shift, no sum overflows all the same: the products'
+// 2-norm is at most N^(1/2) / 4^(T + 1) times the line's (T twiddled passes, the factor 1/4 of the
+// product), and a sum of P of them at most sqrt(P) times that (Cauchy-Schwarz); line_bits keeps it
+// below 2^63 through the inverse passes.
 //
-// Measured against the float64 transforms (1024^2): column pass 1225 -> 240 us per launch of 17
-// fields, flux pass 330 -> 76; float64 step 8.31 -> 5.46 ms by the fixed-point lines alone, 2.32
-// with the node loops and launch shapes that followed. Both integer pipes are half busy (52 and
-// 55%) at 16 warps per SM.
+// Rounding: each product is rounded to the nearest integer up to a quarter unit, inputs are cut off
+// once at 2^(e - B) (B = 54 .. 61). Root-mean-square error of a first derivative against __float128
+// sums, relative to that of the float64 transform by the same radix-16 passes, 4 .. 4096 points: 0.2 to
+// 0.8 for zero-mean noise, 0.0 to 0.45 for smooth and interface profiles, 0.00 to 0.15 for noise about a
+// mean, 0.3 to 0.8 for single points and 0.3 to 1.0 for sharp two-level lines (1.0 at 4096 points); 1.4
+// for a 4096-point line of few-bit values constant but for one point, whose sums float64 holds exactly.
+// Lines of 4 points, whose differences of close values float64 takes exactly: 0.6 to 1.
+//
+// Measured against the float64 transforms (1024^2): column pass 1225 -> 254 us per launch of 17
+// fields, flux pass 330 -> 83; float64 step 8.31 -> 2.40 ms with the node loops and launch shapes.
+// The passes wait for instructions and on latency, both integer pipes about half busy at 16 warps per
+// SM. The mean, the sums and the two shifts are 3 to 7% of a step (1024^2 2.32 -> 2.40 ms, 128 x 256
+// 180 -> 193 us, 64^2 unchanged); without them the errors were 2 to 14 times float64's for sharp levels
+// close to one another, up to 25 times for single points on a constant, from 512 points on, and lines of
+// 4 points constant to 10^-8 kept 9 digits of their derivative.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -153,51 +162,62 @@ template <bool INV, int M> __host__ __device__ __forceinline__ longlong2 w16(lon
 }
 
 // ---- line scaling ------------------------------------------------------------------------
-constexpr int kMaxBits = 58;  // a first radix-16 pass multiplies moduli by up to 16
-// bits of an input point (see above): 62 minus the largest growth of the forward passes
-__host__ __device__ constexpr int input_bits(int log2n) {
-    int g = 0, top = 0, left = log2n;
-    if (log2n >= 4)
-        while (left >= 4) {
+constexpr int kGrid = 61;  // points are cut off at 2^-61 of the line's bound or coarser, before the mean is taken off
+// bits of any line of 2^LOG2N points, LOG2N <= 6 (see line_bits, with l1 = l2 + LOG2N / 2 = LOG2N + 1/2)
+template <int LOG2N> constexpr int kShortBits = LOG2N < 4 ? 62 - LOG2N : 58;
+// Bits B of the input points of a line of more, at least 30. m, l2: log2, relative to 2^e, of bounds of the largest real number and of
+// the 2-norm (the root of the sum of all squares). l1: of the sum of all |Re| + |Im|, or 1/2 less than
+// of N^(1/2) times the 2-norm.
+template <int LOG2N> __host__ __device__ __forceinline__ int line_bits(float m, float l1, float l2) {
+    float best = kGrid;
+    // forward: sums of 2^g points have moduli of at most 2^(m + 1/2 + g), and of at most 2^l1 or
+    // 2^(l1 + 1/2). They may reach 2^62.5, but the sum Re + Im of a quarter of a pass is formed too:
+    // it has a quarter of the first bound, half of the third, but sqrt(2) times the second.
+    int g = 0, twiddled = 0, left = LOG2N;
+    if constexpr (LOG2N >= 4) {
+#pragma unroll
+        for (int p = 0; p < LOG2N / 4; ++p) {
             g += 4;
-            top = g > top ? g : top;
+            best = fminf(best, 62.f + 2 * twiddled - fminf(m + g, l1));
             left -= 4;
-            if (left > 0) g -= 2;  // a twiddled pass
+            if (left > 0) ++twiddled;
         }
-    g += left;
-    top = g > top ? g : top;
-    return 62 - top < kMaxBits ? 62 - top : kMaxBits;
+    }
+    if (left > 0) best = fminf(best, 62.f + 2 * twiddled - fminf(m + g + left, l1));
+    // inverse: the 2-norm of the products times sqrt(P) 4^-t after passes over P points, t of them
+    // twiddled, in half bits
+    int points = LOG2N & 3, t = 0, growth = points;
+    if constexpr (LOG2N >= 4) {
+#pragma unroll
+        for (int p = LOG2N / 4 - 1; p >= 0; --p) {
+            if (LOG2N - 4 - 4 * p > 0) ++t;
+            points += 4;
+            growth = growth > points - 4 * t ? growth : points - 4 * t;
+        }
+    }
+    best = fminf(best, 62.9f - 0.5f * (LOG2N - 4 * twiddled - 4 + growth) - l2);
+    return (int)fmaxf(best, 30.f);  // (NaN lines: any value)
 }
 
 // exponent fields below this (2^-959) count as zero, a line of such values transforms to zero
 constexpr int kMinExp = 64;
 
-// input bits of a line whose sum of |Re| + |Im| is at most 2^c 2^e: a sum of moduli never exceeds
-// 2^c, so sparse lines (fluxes that live on an interface) get more bits than the bound by the maximum
-// alone allows
-template <int LOG2N> __host__ __device__ __forceinline__ int line_bits(int c) {
-    constexpr int base = input_bits(LOG2N);
-    const int b = 62 - c < kMaxBits ? 62 - c : kMaxBits;
-    return b > base ? b : base;
-}
-
-// x 2^(B - e), truncated (the inputs' unit lies below what the passes round at), from the bits of
-// the double x; e = emax - 1022 (emax: the largest exponent field of the line, kMinExp <= emax <=
-// 2046), top = emax + kMaxBits - B
+// x 2^(B - e), truncated, B <= kGrid, from the bits of the double x; e = emax - 1022 (emax: the largest
+// exponent field of the line, kMinExp <= emax <= 2046), top = emax + kGrid - B
 __host__ __device__ __forceinline__ long long from_double(unsigned long long x, int top) {
     const int hi = (int)(x >> 32);
     int d = top - (int)(((unsigned)hi >> 20) & 0x7ffu);
     d = d < 63 ? d : 63;
     const unsigned long long mant =
         ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | (x & 0xffffffffULL);
-    const long long v = (long long)((mant << (kMaxBits - 53)) >> d);
+    const long long v = (long long)((mant << (kGrid - 53)) >> d);
     return hi < 0 ? -v : v;
 }
-// |x| as a float from the high word of its bits, truncated; 0 below the float's normal range,
-// not meaningful above it
-__host__ __device__ __forceinline__ float abs_approx(unsigned long long x) {
-    const int h = (int)((x >> 32) & 0x7fffffffu) - (896 << 20);
-    const unsigned b = h > 0 ? (unsigned)h << 3 : 0u;
+// x 2^-e as a float from the high word of its bits, truncated; off = (emax - 126) 2^20, least the larger
+// of it and 2^20 - 1. 0 for zeros and below the float's normal range.
+__host__ __device__ __forceinline__ float relative(unsigned hi, int off, int least) {
+    const int h = (int)(hi & 0x7fffffffu);
+    const unsigned b = (h > least ? (unsigned)(h - off) << 3 : 0u) | (hi & 0x80000000u);
 #ifdef __CUDA_ARCH__
     return __uint_as_float(b);
 #else

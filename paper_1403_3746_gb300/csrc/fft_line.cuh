@@ -1,9 +1,10 @@
 // Spectral line operators: what the passes call to differentiate a line. Line<float> is the
 // float32 transform of fft_reg.cuh; Line<double> runs the same passes in 64-bit fixed point
-// (fft_fixed.cuh): the line's common exponent from one reduction over its threads, integer points
-// between forward() and inverse(), and float64 values again after it. The spectrum between the two
-// is opaque to the caller (it may be kept with storeF and read back with loadF); Scale carries
-// the line's exponent along with it.
+// (fft_fixed.cuh): the line's common exponent and mean from reductions over its threads, integer
+// points between forward() and inverse(), and float64 values again after it. The spectrum between the
+// two is opaque to the caller (it may be kept with storeF and read back with loadF); Scale carries
+// the line's exponent along with it. Calls go in the order forward, multiply, inverse; a spectrum that
+// is read back goes through multiply and inverse again.
 #pragma once
 #include "fft_reg.cuh"
 
@@ -37,10 +38,10 @@ template <typename R, int LOG2N, bool PK, int CS = 1> struct Line : LineFFT<R, L
         B::template forward<SYNC>(v, buf, t, ax.tw);
         return Scale{};
     }
-    static __device__ __forceinline__ void multiply(CT v[B::E], int t, int order, R c, const Axis<R> &ax, Scale &) {
+    template <class SYNC> static __device__ __forceinline__ void multiply(CT v[B::E], int t, int order, R c, const Axis<R> &ax, Scale &, int) {
         B::multiply(v, t, order, c, ax.k1, ax.k2);
     }
-    template <class SYNC> static __device__ __forceinline__ void inverse(CT v[B::E], CT *buf, int t, const Axis<R> &ax, Scale, int) {
+    template <class SYNC> static __device__ __forceinline__ void inverse(CT v[B::E], CT *buf, int t, const Axis<R> &ax, Scale) {
         B::template inverse<SYNC>(v, buf, t, ax.tw);
     }
 };
@@ -79,86 +80,129 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
         B::store_natural(u, reinterpret_cast<longlong2 *>(buf), t);
     }
 
-    // Whether a line's threads span warps (then the reductions take one CTA barrier each).
-    static __device__ __forceinline__ bool spans_warps(int st) { return GL * st > 32; }
+    // Lines of up to 64 points take as many bits as the largest magnitude allows and keep their mean, and
+    // the multiplier's shift is that of the sum of the points: their errors are at most the float64
+    // transform's as it is, and their passes wait for instructions (64^2 float64 step 155 us, 167 with the
+    // general form).
+    static constexpr bool kShort = LOG2N <= 6;
 
-    // Reduces (a, b) over the line's threads with op, a commutative pair operation. The tree pairs
-    // the bits of t from the lowest up whatever st is, so the result does not depend on the tile
-    // shape even where op rounds (b: a float sum).
-    template <class SYNC, class OP> static __device__ __forceinline__ void reduce(unsigned &a, unsigned &b, int st, OP op) {
+    static __device__ __forceinline__ long long shl(long long a, int n) { return (long long)((unsigned long long)a << n); }
+
+    // Reduces w[0 .. W-1] over the line's threads with op(k, a, b), a commutative operation for each
+    // word k whose neutral element is 0. The tree pairs the bits of t from the lowest up whatever st is, so the
+    // result does not depend on the tile shape even where op rounds (float sums). Where a line's
+    // threads span warps it takes one CTA barrier and words [SLOT, SLOT + W) of the scratch: a call
+    // that may run while another thread still reads the last one's words takes others.
+    static constexpr int kSlots = 5;
+    template <class SYNC, int SLOT, int W, class OP> static __device__ __forceinline__ void reduce(unsigned (&w)[W], int st, OP op) {
+        static_assert(SLOT + W <= kSlots, "scratch words");
         if constexpr (G == 1) return;
         const int tid = threadIdx.x, lane = tid & 31;
         const int n = GL * st;  // threads over which the line's threads spread
         const unsigned mask = n >= 32 ? 0xffffffffu : ((1u << n) - 1u) << (lane & ~(n - 1));
-        for (int off = st; off < 32 && off < n; off <<= 1) {
-            const unsigned oa = __shfl_xor_sync(mask, a, off), ob = __shfl_xor_sync(mask, b, off);
-            op(a, b, oa, ob);
-        }
+        for (int off = st; off < 32 && off < n; off <<= 1)
+#pragma unroll
+            for (int k = 0; k < W; ++k) w[k] = op(k, w[k], __shfl_xor_sync(mask, w[k], off));
         if (n > 32) {
-            __shared__ uint2 part[128];  // one entry per warp and line
-            const int nw = n >> 5, w = tid >> 5, l = tid & (st - 1);
-            if (lane < st) part[w * st + l] = make_uint2(a, b);
+            // one entry per warp and line: a line spans at most 8 warps, and at most 16 lines of a tile share them
+            unsigned(*part)[kPart] = scratch();
+            const int nw = n >> 5, wp = tid >> 5, l = tid & (st - 1);
+            if (lane < st) {
+#pragma unroll
+                for (int k = 0; k < W; ++k) part[SLOT + k][wp * st + l] = w[k];
+            }
             SYNC::run();
-            const int w0 = w & ~(nw - 1);
-            uint2 r[8];  // a line spans at most 8 warps; (0, 0) is neutral
+            const int w0 = wp & ~(nw - 1);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) r[i] = i < nw ? part[(w0 + i) * st + l] : make_uint2(0u, 0u);
+            for (int k = 0; k < W; ++k) {
+                unsigned r[8];
 #pragma unroll
-            for (int d = 1; d < 8; d <<= 1)
+                for (int i = 0; i < 8; ++i) r[i] = i < nw ? part[SLOT + k][(w0 + i) * st + l] : 0u;
 #pragma unroll
-                for (int i = 0; i + d < 8; i += 2 * d) op(r[i].x, r[i].y, r[i + d].x, r[i + d].y);
-            a = r[0].x;
-            b = r[0].y;
+                for (int d = 1; d < 8; d <<= 1)
+#pragma unroll
+                    for (int i = 0; i + d < 8; i += 2 * d) r[i] = op(k, r[i], r[i + d]);
+                w[k] = r[0];
+            }
         }
         if constexpr (CS > 1) {  // the other CTAs' parts of the line, through distributed shared memory
-            __shared__ __align__(16) uint2 cpart[CS * 32];
+            __shared__ unsigned cpart[W][CS * 32];
             const int l = tid & (st - 1);
             cluster_barrier();
             if (tid < st) {
 #pragma unroll
-                for (int r = 0; r < CS; ++r) {
-                    const uint32_t p = cluster_map(&cpart[cluster_rank() * 32 + l], r);
-                    asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(p), "r"(a), "r"(b) : "memory");
-                }
+                for (int r = 0; r < CS; ++r)
+#pragma unroll
+                    for (int k = 0; k < W; ++k) {
+                        const uint32_t p = cluster_map(&cpart[k][cluster_rank() * 32 + l], r);
+                        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(p), "r"(w[k]) : "memory");
+                    }
             }
             cluster_barrier();
-            uint2 r[CS];
 #pragma unroll
-            for (int i = 0; i < CS; ++i) r[i] = cpart[i * 32 + l];
+            for (int k = 0; k < W; ++k) {
+                unsigned r[CS];
 #pragma unroll
-            for (int d = 1; d < CS; d <<= 1)
+                for (int i = 0; i < CS; ++i) r[i] = cpart[k][i * 32 + l];
 #pragma unroll
-                for (int i = 0; i + d < CS; i += 2 * d) op(r[i].x, r[i].y, r[i + d].x, r[i + d].y);
-            a = r[0].x;
-            b = r[0].y;
+                for (int d = 1; d < CS; d <<= 1)
+#pragma unroll
+                    for (int i = 0; i + d < CS; i += 2 * d) r[i] = op(k, r[i], r[i + d]);
+                w[k] = r[0];
+            }
         }
+    }
+    static constexpr int kPart = 128;
+    static __device__ __forceinline__ unsigned (*scratch())[kPart] {
+        __shared__ unsigned part[kSlots][kPart];
+        return part;
     }
 
     template <class SYNC> static __device__ __forceinline__ Scale forward(CT v[E], CT *buf, int t, const Axis<double> &ax, int st) {
         longlong2 u[E];
         get(u, v);
-        // the line's largest magnitude (high words order as the values do) and the sum of all
-        unsigned top = 0;
-        float l1 = 0.f;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const unsigned hx = (unsigned)(u[e].x >> 32) & 0x7fffffffu, hy = (unsigned)(u[e].y >> 32) & 0x7fffffffu;
-            top = max(top, max(hx, hy));
-            l1 += fixed::abs_approx(u[e].x) + fixed::abs_approx(u[e].y);
-        }
-        unsigned l1b = __float_as_uint(l1);
-        reduce<SYNC>(top, l1b, st, [](unsigned &a, unsigned &b, unsigned oa, unsigned ob) {
-            a = max(a, oa);
-            b = __float_as_uint(__fadd_rn(__uint_as_float(b), __uint_as_float(ob)));
-        });
-        const int emax = (int)(top >> 20);
-        // the sum counts where neither it nor its terms leave the float range: 2^c 2^e bounds it
-        const int c = emax > 930 && emax < 1120 ? (int)(l1b >> 23) - 126 - (emax - 1022) : 62;
-        const int bits = fixed::line_bits<LOG2N>(c);
-        const int shift = emax + fixed::kMaxBits - bits;
+        // the line's largest magnitude (high words order as the values do)
+        unsigned top[1] = {0};
 #pragma unroll
         for (int e = 0; e < E; ++e)
-            u[e] = fixed::mk2(fixed::from_double((unsigned long long)u[e].x, shift), fixed::from_double((unsigned long long)u[e].y, shift));
+            top[0] = max(top[0], max((unsigned)(u[e].x >> 32) & 0x7fffffffu, (unsigned)(u[e].y >> 32) & 0x7fffffffu));
+        reduce<SYNC, 0>(top, st, [](int, unsigned a, unsigned b) { return max(a, b); });
+        const int emax = (int)(top[0] >> 20);
+        int bits = fixed::kShortBits<LOG2N>;
+        long long cx = 0, cy = 0;
+        if constexpr (!kShort) {
+            // sums relative to it
+            const int off = (emax - 126) << 20, least = max(off, (1 << 20) - 1);
+            float l1 = 0.f, l2 = 0.f, sx = 0.f, sy = 0.f;  // magnitudes, squares, the two fields' values
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const float x = fixed::relative((unsigned)(u[e].x >> 32), off, least), y = fixed::relative((unsigned)(u[e].y >> 32), off, least);
+                l1 += fabsf(x) + fabsf(y);
+                l2 = fmaf(x, x, fmaf(y, y, l2));
+                sx += x;
+                sy += y;
+            }
+            unsigned sums[4] = {__float_as_uint(l1), __float_as_uint(l2), __float_as_uint(sx), __float_as_uint(sy)};
+            reduce<SYNC, 1>(sums, st, [](int, unsigned a, unsigned b) { return __float_as_uint(__fadd_rn(__uint_as_float(a), __uint_as_float(b))); });
+            // bits with the points as they are, and with the mean taken out: the sum of squares about it (the
+            // truncated values' relative error, 2^-19, covered) bounds the largest deviation and any sum of P
+            // points; a hundredth covers the rounding of sums and logarithms
+            const float s2 = __uint_as_float(sums[1]), mx = __uint_as_float(sums[2]) * (1.f / B::N), my = __uint_as_float(sums[3]) * (1.f / B::N);
+            const float d2 = fmaxf(s2 - B::N * (mx * mx + my * my), 0.f) + s2 * 0x1p-16f;
+            const float ld = 0.5f * __log2f(d2) + 0.01f;
+            bits = fixed::line_bits<LOG2N>(0.f, __log2f(__uint_as_float(sums[0])) + 0.01f, 0.5f * __log2f(s2) + 0.01f);
+            const int about = fixed::line_bits<LOG2N>(fminf(1.f, ld), ld + 0.5f * (LOG2N - 1), ld);
+            if (about > bits) {
+                bits = about;
+                cx = shl((long long)__float2int_rn(mx * 0x1p30f), bits - 30);
+                cy = shl((long long)__float2int_rn(my * 0x1p30f), bits - 30);
+            }
+        }
+        const int shift = emax + fixed::kGrid - bits;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            u[e] = fixed::mk2(fixed::from_double((unsigned long long)u[e].x, shift) - cx,
+                              fixed::from_double((unsigned long long)u[e].y, shift) - cy);
         B::template forward<SYNC>(u, reinterpret_cast<longlong2 *>(buf), t, ax.tw);
         put(v, u);
         Scale s;
@@ -166,46 +210,68 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
         return s;
     }
 
-    // v <- d^order c v
-    static __device__ __forceinline__ void multiply(CT v[E], int t, int order, double c, const Axis<double> &ax, Scale &s) {
+    // v <- d^order c v, as integers whose magnitudes sum to just below 2^63 where that is an upward shift
+    template <class SYNC> static __device__ __forceinline__ void multiply(CT v[E], int t, int order, double c, const Axis<double> &ax, Scale &s, int st) {
         longlong2 u[E];
         get(u, v);
         const long long *k = order == 1 ? ax.k1 : ax.k2;
+        int pre, post;  // shifts of the points and of the products
+        if constexpr (G == 1) {  // a whole line: the points' sum in units of 2^6, rounded up, kept below 2^62
+            unsigned long long sum = 1;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const long long x = u[e].x ^ (u[e].x >> 63), y = u[e].y ^ (u[e].y >> 63);
+                if (__ldg(k + e) != 0) sum += ((unsigned long long)x >> 6) + ((unsigned long long)y >> 6) + 2;
+            }
+            const int lz = fixed::clz64(sum);
+            pre = max(lz - 8, 0);
+            post = min(max(lz - 6, 0), 2);
+        } else if constexpr (kShort) {  // the points' sum in units of 2^40
+            unsigned r[1] = {2 * E};
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int hx = fixed::hi32(u[e].x), hy = fixed::hi32(u[e].y);
+                if (__ldg(k + G * e + t) != 0) r[0] += ((unsigned)(hx ^ (hx >> 31)) >> 8) + ((unsigned)(hy ^ (hy >> 31)) >> 8);
+            }
+            reduce<SYNC, 0>(r, st, [](int, unsigned a, unsigned b) { return a + b; });
+            const int total = __clz((int)(r[0] + 2u * B::N)) - 9;
+            pre = max(total, 0);
+            post = min(max(total + 2, 0), 2);
+        } else {  // the products' sum in units of 2^36 (two more for each that is cut off); the points' highest bit
+            unsigned r[2] = {0, 4 * E};
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const long long w = __ldg(k + G * e + t);
+                const unsigned hx = (unsigned)(fixed::hi32(u[e].x) ^ (fixed::hi32(u[e].x) >> 31)), hy = (unsigned)(fixed::hi32(u[e].y) ^ (fixed::hi32(u[e].y) >> 31));
+                if (w != 0) {
+                    const unsigned wh = ((unsigned)abs(fixed::hi32(w)) >> 4) + 1;
+                    r[0] |= hx | hy;
+                    r[1] += __umulhi(hx, wh) + __umulhi(hy, wh);
+                }
+            }
+            reduce<SYNC, 0>(r, st, [](int k, unsigned a, unsigned b) { return k == 0 ? a | b : a + b; });
+            const int total = __clz((int)(r[1] + 2u * B::N)) - 5;
+            pre = max(min(total, __clz((int)r[0]) - 2), 0);
+            post = max(total - pre, 0);
+        }
         const bool unit = c == 1.0;
         const fixed::Factor f = fixed::factor((unsigned long long)__double_as_longlong(c));
-        if (s.ex != kNan && s.ex != kZero) s.ex += 2 + (order == 1 ? ax.p1 : ax.p2) + (unit ? 0 : f.ex);
+        if (s.ex != kNan && s.ex != kZero) s.ex += 2 + (order == 1 ? ax.p1 : ax.p2) + (unit ? 0 : f.ex) - pre - post;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             long long w = __ldg(k + G * e + t);
             if (!unit) w = fixed::balance(fixed::mulhi(fixed::hi32(w), fixed::lo32(w), fixed::hi32(f.m), fixed::lo32(f.m)) << 2);
-            const long long x = fixed::mulhi(u[e].x, w), y = fixed::mulhi(u[e].y, w);
+            const long long x = shl(fixed::mulhi(shl(u[e].x, pre), w), post), y = shl(fixed::mulhi(shl(u[e].y, pre), w), post);
             u[e] = order == 1 ? fixed::mk2(-y, x) : fixed::mk2(x, y);
         }
         put(v, u);
     }
 
-    template <class SYNC> static __device__ __forceinline__ void inverse(CT v[E], CT *buf, int t, const Axis<double> &ax, Scale s, int st) {
+    template <class SYNC> static __device__ __forceinline__ void inverse(CT v[E], CT *buf, int t, const Axis<double> &ax, Scale s) {
         longlong2 u[E];
         get(u, v);
-        // the sum of the spectrum's magnitudes in units of 2^40, rounded up: the shift that brings
-        // it just below 2^63
-        unsigned sum = 0, zero = 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int hx = fixed::hi32(u[e].x), hy = fixed::hi32(u[e].y);
-            sum += ((unsigned)(hx ^ (hx >> 31)) >> 8) + ((unsigned)(hy ^ (hy >> 31)) >> 8);
-        }
-        reduce<SYNC>(sum, zero, st, [](unsigned &a, unsigned &b, unsigned oa, unsigned ob) {
-            a += oa;
-            b |= ob;
-        });
-        int sh = __clz((int)(sum + 2u * B::N)) - 9;
-        sh = sh > 0 ? sh : 0;
-#pragma unroll
-        for (int e = 0; e < E; ++e)
-            u[e] = fixed::mk2((long long)((unsigned long long)u[e].x << sh), (long long)((unsigned long long)u[e].y << sh));
         B::template inverse<SYNC>(u, reinterpret_cast<longlong2 *>(buf), t, ax.tw);
-        const int ex = s.ex + 2 * T - sh;
+        const int ex = s.ex + 2 * T;
         if (ex > -960 && ex < 950) {
 #pragma unroll
             for (int e = 0; e < E; ++e)
@@ -226,10 +292,14 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
         }
     }
 
-    // barriers only (see LineFFT): the reductions of a line that spans warps add one each
+    // barriers only (see LineFFT), of forward and of multiply and inverse: the reductions of a line that
+    // spans warps add one each
     template <class SYNC> static __device__ __forceinline__ void idle_forward() {
         static_assert(CS == 1, "float64 rows are not split over clusters");
-        if constexpr (GL > 32) SYNC::run();
+        if constexpr (GL > 32) {
+            SYNC::run();
+            SYNC::run();
+        }
         B::template idle_forward<SYNC>();
     }
     template <class SYNC> static __device__ __forceinline__ void idle_inverse() {

@@ -176,8 +176,8 @@ __global__ void __launch_bounds__(PassThreads<R>::value, PassThreads<R>::min_blo
         for (int e = 0; e < F::E; ++e) v[e] = st[(size_t)(t + F::G * e) * L + l];  // row t + G e, columns 2l, 2l+1
         CT *buf = st + l * col_line_stride(LOG2N, sizeof(R), 1);
         typename F::Scale sc = F::template forward<reg::SyncCta>(v, buf, t, c.ay, L);
-        F::multiply(v, t, jb.order, jb.c, c.ay, sc);
-        F::template inverse<reg::SyncCta>(v, buf, t, c.ay, sc, L);
+        F::template multiply<reg::SyncCta>(v, t, jb.order, jb.c, c.ay, sc, L);
+        F::template inverse<reg::SyncCta>(v, buf, t, c.ay, sc);
         const size_t rso = (size_t)(jb.ld_out >> 1), rsi = (size_t)(jb.ld_in >> 1);
         CT *out = reinterpret_cast<CT *>(jb.out + (size_t)z_of(it) * c.ny * jb.ld_out + tile_of(it) * W + 2 * l);
         const CT *inp = reinterpret_cast<const CT *>(jb.in + (size_t)z_of(it) * c.ny * jb.ld_in + tile_of(it) * W + 2 * l);

@@ -142,8 +142,8 @@ __global__ void __launch_bounds__(256, 2) rho64_row_kernel(double *r64, const __
     for (int order = 1; order <= 2; ++order) {
         typename F::Scale sc = sc0;
         if (order == 2) F::loadF(v, spec, t);
-        F::multiply(v, t, order, 1.0, ax, sc);
-        F::template inverse<reg::SyncCta>(v, buf, t, ax, sc, 1);
+        F::template multiply<reg::SyncCta>(v, t, order, 1.0, ax, sc, 1);
+        F::template inverse<reg::SyncCta>(v, buf, t, ax, sc);
         const int o = (order == 1 ? R64_RX : R64_RXX) * NX + t;
 #pragma unroll
         for (int e = 0; e < E; ++e) row[o + G * e] = v[e].x, row1[o + G * e] = v[e].y;
@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(MaxThreads<R>::value, MaxThreads<R>::min_block
     }
     CT *buf = sb + (size_t)slot * F::STRIDE;
     typename F::Scale sc = F::template forward<reg::SyncCta>(v, buf, t, a.ax, 1);
-    F::multiply(v, t, a.order == 2 ? 2 : 1, R(1), a.ax, sc);
-    F::template inverse<reg::SyncCta>(v, buf, t, a.ax, sc, 1);
+    F::template multiply<reg::SyncCta>(v, t, a.order == 2 ? 2 : 1, R(1), a.ax, sc, 1);
+    F::template inverse<reg::SyncCta>(v, buf, t, a.ax, sc);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const size_t g = row + t + G * e;

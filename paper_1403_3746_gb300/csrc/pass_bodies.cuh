@@ -41,8 +41,8 @@ __device__ __forceinline__ void col_tile(const ColArgs<R> &a, int jobi, int z, i
     for (int e = 0; e < F::E; ++e) v[e] = __ldcg(in + (size_t)(t + F::G * e) * rsi);  // L2 only: single use
     CT *buf = sbuf + l * col_line_stride(LOG2N, sizeof(R), CS);
     typename F::Scale sc = F::template forward<reg::SyncCta>(v, buf, t, a.ay, L);
-    F::multiply(v, t, job.order, job.c, a.ay, sc);
-    F::template inverse<reg::SyncCta>(v, buf, t, a.ay, sc, L);
+    F::template multiply<reg::SyncCta>(v, t, job.order, job.c, a.ay, sc, L);
+    F::template inverse<reg::SyncCta>(v, buf, t, a.ay, sc);
     if constexpr (ACC) {  // out = in + result; each position is read and written by this thread only
 #pragma unroll
         for (int e = 0; e < F::E; ++e) {
@@ -186,8 +186,8 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
                     sc0 = sc;
                 }
             }
-            F::multiply(v, t, it == 1 ? 2 : 1, R(1), a.ax, sc);
-            F::template inverse<reg::SyncCta>(v, O, t, a.ax, sc, 1);
+            F::template multiply<reg::SyncCta>(v, t, it == 1 ? 2 : 1, R(1), a.ax, sc, 1);
+            F::template inverse<reg::SyncCta>(v, O, t, a.ax, sc);
             if (it < 2) {
                 reg::cta_barrier();
 #pragma unroll
@@ -787,8 +787,8 @@ __device__ __forceinline__ void update_rows(const UpdateArgs<R> &a, const Update
 #pragma unroll
                 for (int e = 0; e < E; ++e) v[e] = reg::mk<R>(ldcg(fa + t + G * e), ldcg(fb + t + G * e));
                 typename F::Scale sc = F::template forward<reg::SyncCta>(v, buf, t, a.ax, 1);
-                F::multiply(v, t, 1, a.cx[p], a.ax, sc);  // -h v_x folded in
-                F::template inverse<reg::SyncCta>(v, buf, t, a.ax, sc, 1);
+                F::template multiply<reg::SyncCta>(v, t, 1, a.cx[p], a.ax, sc, 1);  // -h v_x folded in
+                F::template inverse<reg::SyncCta>(v, buf, t, a.ax, sc);
                 if constexpr (CS == 1) reg::cta_barrier();  // (a split inverse ends with a cluster barrier)
                 F::store_natural(v, buf, t);
             } else {
