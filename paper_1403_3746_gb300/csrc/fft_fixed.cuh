@@ -39,6 +39,7 @@
 // 4 points constant to 10^-8 kept 9 digits of their derivative.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 
 namespace lbm {
 namespace fixed {
@@ -242,6 +243,29 @@ __host__ __device__ __forceinline__ unsigned long long to_double(long long y, in
     const unsigned hi = (unsigned)(v >> 32) + ((unsigned)(ex + 1023 + 62 - lz) << 20);
     const unsigned long long r = ((unsigned long long)(hi | ((unsigned)(y >> 32) & 0x80000000u)) << 32) | (v & 0xffffffffULL);
     return m ? r : 0ULL;
+}
+
+// Sum of 16 floats (their bits) as the bits of a double: exact but for what lies below 2^-58 of the
+// largest (less than one rounding of a float64 sum), then rounded once. False, and no sum, where the
+// largest is below 2^-63, infinite or NaN.
+__host__ __device__ __forceinline__ bool sum16(const unsigned f[16], unsigned long long &bits) {
+    unsigned top = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const unsigned a = f[i] & 0x7fffffffu;
+        top = a > top ? a : top;
+    }
+    const int et = (int)(top >> 23);  // every |f| < 2^(et - 126)
+    long long sum = 0;                // unit 2^(et - 185): 16 values below 2^59
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int sh = (int)((f[i] >> 23) & 0xffu) - et + 35;
+        const unsigned m = (f[i] & 0x7fffffu) | 0x800000u;
+        const unsigned long long v = sh >= 0 ? (unsigned long long)m << (sh & 63) : (unsigned long long)(m >> (-sh < 31 ? -sh : 31));
+        sum += (int)f[i] < 0 ? -(long long)v : (long long)v;
+    }
+    bits = to_double(sum, et - 185);
+    return et >= 64 && et < 255;
 }
 
 // A real factor c = m 2^ex as a fixed-point number m 2^62 (|m| in [1/2, 1)) in balanced halves

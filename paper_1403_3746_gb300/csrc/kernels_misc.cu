@@ -85,35 +85,23 @@ __global__ void moments_kernel(const __grid_constant__ MomArgs a) {
     }
 }
 
-// LBM_MIXED_RHO64: rho of every node as the sum of its 16 stored float32 values, exact to 2^-56 and
-// then rounded once to float64. The sum runs in 64-bit integers of unit 2^-56 (|f| < 4), because the
-// 31 conversions and additions of the float64 form take 16 clocks of an SM's float64 unit per node
-// (with the one-launch row pass below, 1024^2: 188 -> 120 us per stage for the whole chain); nodes
-// with a larger, infinite or NaN value take that form.
+// LBM_MIXED_RHO64: rho of every node as the sum of its 16 stored float32 values (fixed::sum16). In
+// integers, because the 31 conversions and additions of a float64 sum take 16 clocks of an SM's float64
+// unit per node (with the one-launch row pass below, 1024^2: 188 -> 119 us per stage for the whole chain).
 __global__ void __launch_bounds__(256) rho64_kernel(const float *f, double *r64, int nx, int ny) {
     const long long n = (long long)nx * ny;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < n;
          g += (long long)gridDim.x * blockDim.x) {
         const long long y = g / nx, x = g - y * nx;
         const float *fn = f + y * NF_F * nx + x;
-        unsigned bits[16], top = 0;
-        long long sum = 0;
+        unsigned bits[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) bits[i] = __float_as_uint(__ldcg(fn + i * nx));
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const unsigned a = bits[i] & 0x7fffffffu;
-            top = max(top, a);
-            const int sh = (int)(a >> 23) - 94;  // unit 2^-56
-            const unsigned m = (a & 0x7fffffu) | 0x800000u;
-            const unsigned long long v = sh >= 0 ? (unsigned long long)m << (sh & 63) : (unsigned long long)(m >> min(-sh, 31));
-            sum += (int)bits[i] < 0 ? -(long long)v : (long long)v;
-        }
-        double s;
-        if (top < 0x40800000u) {  // every |f| < 4
-            s = __longlong_as_double((long long)fixed::to_double(sum, -56));
+        unsigned long long sum;
+        double s = 0.0;
+        if (fixed::sum16(bits, sum)) {
+            s = __longlong_as_double((long long)sum);
         } else {
-            s = 0.0;
 #pragma unroll
             for (int i = 0; i < 16; ++i) s += (double)__uint_as_float(bits[i]);
         }
