@@ -4,14 +4,15 @@
 // 32-bit multiply-adds (measured: add.s64 64 per clock and SM, mul.wide.s32 60, fma.f64 2.0). A
 // complex butterfly addition is four integer instructions instead of two float64 ones that take
 // 32 times their slots, so the float64 lines are transformed as 64-bit integers that share one
-// exponent per complex line (block floating point).
+// exponent per real line (block floating point).
 //
-// Scaling of a line of N = 2^LOG2N points. Let 2^e bound the magnitude of the line's 2 N real
-// numbers (from their exponents). Point x enters as trunc((x - c) 2^(B - e)). c is the line's mean,
-// taken out where that leaves more bits: every multiplier is zero at index 0, so a constant never
-// reaches the result. Every radix-16 pass that has outer twiddles ends (forward) or begins (inverse)
-// with a factor 1/4, which the high half of the product with a root scaled to 2^62 gives for free. B is
-// the largest value (line_bits) for which no sum can reach 2^63: a pass multiplies the largest
+// Scaling of a complex line of N = 2^LOG2N points, which is two real lines. Let 2^e bound the
+// magnitude of a real line's numbers (from their exponents; each of the two has its own). Point x
+// enters as trunc((x - c) 2^(B - e)). c is the line's mean, taken out where that leaves more bits:
+// every multiplier is zero at index 0, so a constant never reaches the result. Every radix-16 pass
+// that has outer twiddles ends (forward) or begins (inverse) with a factor 1/4, which the high half of
+// the product with a root scaled to 2^62 gives for free. B is the largest value (line_bits) for
+// which no sum can reach 2^63: a pass multiplies the largest
 // modulus by at most the points it has summed, and no sum of points passes the sum of all moduli.
 //
 // The spectrum is shifted up before it meets the multiplier, as far as its largest entry with a
@@ -24,19 +25,20 @@
 //
 // Rounding: each product is rounded to the nearest integer up to a quarter unit, inputs are cut off
 // once at 2^(e - B) (B = 54 .. 61). Root-mean-square error of a first derivative against __float128
-// sums, relative to that of the float64 transform by the same radix-16 passes, 4 .. 4096 points: 0.2 to
-// 0.8 for zero-mean noise, 0.0 to 0.45 for smooth and interface profiles, 0.00 to 0.15 for noise about a
-// mean, 0.3 to 0.8 for single points and 0.3 to 1.0 for sharp two-level lines (1.0 at 4096 points); 1.4
-// for a 4096-point line of few-bit values constant but for one point, whose sums float64 holds exactly.
-// Lines of 4 points, whose differences of close values float64 takes exactly: 0.6 to 1.
+// sums, relative to that of the float64 transform by the same radix-16 passes, 4 .. 4096 points: 0.3 to
+// 0.8 for zero-mean noise, 0.0 to 0.5 for smooth and interface profiles and for noise about a mean, 0.3
+// to 0.8 for single points, 0.1 to 1.05 for sharp two-level lines (the most at 4096 points); 1.4 for a
+// 4096-point line of few-bit values constant but for one point, whose sums float64 holds exactly. Lines
+// of 4 points, whose differences of close values float64 takes exactly: 0.4 to 1.
 //
 // Measured against the float64 transforms (1024^2): column pass 1225 -> 254 us per launch of 17
-// fields, flux pass 330 -> 83; float64 step 8.31 -> 2.40 ms with the node loops and launch shapes.
+// fields, flux pass 330 -> 83; float64 step 8.31 -> 2.44 ms with the node loops and launch shapes.
 // The passes wait for instructions and on latency, both integer pipes about half busy at 16 warps per
-// SM. The mean, the sums and the two shifts are 3 to 7% of a step (1024^2 2.32 -> 2.40 ms, 128 x 256
-// 180 -> 193 us, 64^2 unchanged); without them the errors were 2 to 14 times float64's for sharp levels
-// close to one another, up to 25 times for single points on a constant, from 512 points on, and lines of
-// 4 points constant to 10^-8 kept 9 digits of their derivative.
+// SM. The two exponents, the mean, the sums and the two shifts are 4 to 7% of a step (1024^2 2.31 -> 2.44
+// ms, 128 x 256 180 -> 193 us, 64^2 unchanged); without them the errors were 2 to 14 times float64's for
+// sharp levels close to one another, up to 25 times for single points on a constant, from 512 points
+// on, lines of 4 points constant to 10^-8 kept 9 digits of their derivative, and a line 10^-9 times its
+// partner 8.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>

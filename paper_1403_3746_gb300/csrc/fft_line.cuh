@@ -50,9 +50,10 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
     using B = LineFFT<long long, LOG2N, false, CS>;
     typedef double2 CT;
     static constexpr int E = B::E, G = B::G, GL = B::GL, T = B::TWIDDLED;
-    // values are integers times 2^ex; all of them NaN, or all zero, where ex is one of these
+    // the real and the imaginary parts, which are two real lines, are integers times 2^ex and 2^ey; all of
+    // them NaN, or all zero, where these lie near kNan and kZero
     struct Scale {
-        int ex;
+        int ex, ey;
     };
     static constexpr int kNan = 1 << 20, kZero = -(1 << 20);
 
@@ -93,7 +94,7 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
     // result does not depend on the tile shape even where op rounds (float sums). Where a line's
     // threads span warps it takes one CTA barrier and words [SLOT, SLOT + W) of the scratch: a call
     // that may run while another thread still reads the last one's words takes others.
-    static constexpr int kSlots = 5;
+    static constexpr int kSlots = 6;
     template <class SYNC, int SLOT, int W, class OP> static __device__ __forceinline__ void reduce(unsigned (&w)[W], int st, OP op) {
         static_assert(SLOT + W <= kSlots, "scratch words");
         if constexpr (G == 1) return;
@@ -161,29 +162,32 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
     template <class SYNC> static __device__ __forceinline__ Scale forward(CT v[E], CT *buf, int t, const Axis<double> &ax, int st) {
         longlong2 u[E];
         get(u, v);
-        // the line's largest magnitude (high words order as the values do)
-        unsigned top[1] = {0};
+        // the two lines' largest magnitudes (high words order as the values do): each has its own exponent,
+        // so that neither loses bits to a larger partner
+        unsigned top[2] = {0, 0};
 #pragma unroll
-        for (int e = 0; e < E; ++e)
-            top[0] = max(top[0], max((unsigned)(u[e].x >> 32) & 0x7fffffffu, (unsigned)(u[e].y >> 32) & 0x7fffffffu));
+        for (int e = 0; e < E; ++e) {
+            top[0] = max(top[0], (unsigned)(u[e].x >> 32) & 0x7fffffffu);
+            top[1] = max(top[1], (unsigned)(u[e].y >> 32) & 0x7fffffffu);
+        }
         reduce<SYNC, 0>(top, st, [](int, unsigned a, unsigned b) { return max(a, b); });
-        const int emax = (int)(top[0] >> 20);
+        const int ex = (int)(top[0] >> 20), ey = (int)(top[1] >> 20);
         int bits = fixed::kShortBits<LOG2N>;
         long long cx = 0, cy = 0;
         if constexpr (!kShort) {
-            // sums relative to it
-            const int off = (emax - 126) << 20, least = max(off, (1 << 20) - 1);
+            // sums relative to them
+            const int ox = (ex - 126) << 20, oy = (ey - 126) << 20, least_x = max(ox, (1 << 20) - 1), least_y = max(oy, (1 << 20) - 1);
             float l1 = 0.f, l2 = 0.f, sx = 0.f, sy = 0.f;  // magnitudes, squares, the two fields' values
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                const float x = fixed::relative((unsigned)(u[e].x >> 32), off, least), y = fixed::relative((unsigned)(u[e].y >> 32), off, least);
+                const float x = fixed::relative((unsigned)(u[e].x >> 32), ox, least_x), y = fixed::relative((unsigned)(u[e].y >> 32), oy, least_y);
                 l1 += fabsf(x) + fabsf(y);
                 l2 = fmaf(x, x, fmaf(y, y, l2));
                 sx += x;
                 sy += y;
             }
             unsigned sums[4] = {__float_as_uint(l1), __float_as_uint(l2), __float_as_uint(sx), __float_as_uint(sy)};
-            reduce<SYNC, 1>(sums, st, [](int, unsigned a, unsigned b) { return __float_as_uint(__fadd_rn(__uint_as_float(a), __uint_as_float(b))); });
+            reduce<SYNC, 2>(sums, st, [](int, unsigned a, unsigned b) { return __float_as_uint(__fadd_rn(__uint_as_float(a), __uint_as_float(b))); });
             // bits with the points as they are, and with the mean taken out: the sum of squares about it (the
             // truncated values' relative error, 2^-19, covered) bounds the largest deviation and any sum of P
             // points; a hundredth covers the rounding of sums and logarithms
@@ -198,15 +202,17 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
                 cy = shl((long long)__float2int_rn(my * 0x1p30f), bits - 30);
             }
         }
-        const int shift = emax + fixed::kGrid - bits;
+        const int g = fixed::kGrid - bits, shift_x = ex < fixed::kMinExp ? 1 << 12 : ex + g, shift_y = ey < fixed::kMinExp ? 1 << 12 : ey + g;
 #pragma unroll
         for (int e = 0; e < E; ++e)
-            u[e] = fixed::mk2(fixed::from_double((unsigned long long)u[e].x, shift) - cx,
-                              fixed::from_double((unsigned long long)u[e].y, shift) - cy);
+            u[e] = fixed::mk2(fixed::from_double((unsigned long long)u[e].x, shift_x) - cx,
+                              fixed::from_double((unsigned long long)u[e].y, shift_y) - cy);
         B::template forward<SYNC>(u, reinterpret_cast<longlong2 *>(buf), t, ax.tw);
         put(v, u);
+        const bool bad = max(ex, ey) == 0x7ff;
         Scale s;
-        s.ex = emax == 0x7ff ? kNan : emax < fixed::kMinExp ? kZero : emax - 1022 - bits + 2 * T;
+        s.ex = bad ? kNan : ex < fixed::kMinExp ? kZero : ex - 1022 - bits + 2 * T;
+        s.ey = bad ? kNan : ey < fixed::kMinExp ? kZero : ey - 1022 - bits + 2 * T;
         return s;
     }
 
@@ -256,7 +262,9 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
         }
         const bool unit = c == 1.0;
         const fixed::Factor f = fixed::factor((unsigned long long)__double_as_longlong(c));
-        if (s.ex != kNan && s.ex != kZero) s.ex += 2 + (order == 1 ? ax.p1 : ax.p2) + (unit ? 0 : f.ex) - pre - post;
+        const int scale = 2 + (order == 1 ? ax.p1 : ax.p2) + (unit ? 0 : f.ex) - pre - post;
+        s.ex += scale;
+        s.ey += scale;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             long long w = __ldg(k + G * e + t);
@@ -271,24 +279,24 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
         longlong2 u[E];
         get(u, v);
         B::template inverse<SYNC>(u, reinterpret_cast<longlong2 *>(buf), t, ax.tw);
-        const int ex = s.ex + 2 * T;
-        if (ex > -960 && ex < 950) {
+        const int ex = s.ex + 2 * T, ey = s.ey + 2 * T;
+        if (min(ex, ey) > -960 && max(ex, ey) < 950) {
 #pragma unroll
             for (int e = 0; e < E; ++e)
-                u[e] = fixed::mk2((long long)fixed::to_double(u[e].x, ex), (long long)fixed::to_double(u[e].y, ex));
+                u[e] = fixed::mk2((long long)fixed::to_double(u[e].x, ex), (long long)fixed::to_double(u[e].y, ey));
             put(v, u);
         } else {  // NaN and zero lines, and results near the ends of the float64 range
-            const bool bad = s.ex == kNan;
+            const bool bad = ex > kNan / 2;
             auto pow2 = [](int k) { return __longlong_as_double((long long)(k + 1023) << 52); };
-            const double p = ex < 0 ? pow2(-900) : pow2(900);
-            const double q = ex < 0 ? pow2(max(ex + 900, -1022)) : pow2(min(ex - 900, 1000));
+            auto value = [&](long long y, int k) {
+                const double p = k < 0 ? pow2(-900) : pow2(900);
+                const double q = k < 0 ? pow2(max(k + 900, -1022)) : pow2(min(k - 900, 1000));
+                return __longlong_as_double((long long)fixed::to_double(y, 0)) * p * q;
+            };
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const double x = __longlong_as_double((long long)fixed::to_double(u[e].x, 0)) * p * q;
-                const double y = __longlong_as_double((long long)fixed::to_double(u[e].y, 0)) * p * q;
+            for (int e = 0; e < E; ++e)
                 v[e] = bad ? make_double2(__longlong_as_double(0x7ff8000000000000LL), __longlong_as_double(0x7ff8000000000000LL))
-                           : make_double2(x, y);
-            }
+                           : make_double2(value(u[e].x, ex), value(u[e].y, ey));
         }
     }
 

@@ -69,6 +69,16 @@ def exact(lines, n, where):
     return np.stack([h @ col[(r - j) % n] for r in where], axis=1)
 
 
+def difference(f, dt):
+    """f - f after one advection-only Euler step."""
+    ny, nx = f.shape[1:]
+    with lbm.Simulation(nx, ny, lbm.default_params(flags=FLAGS, dt=dt, tau=1.0, dx=1.0, dy=1.0)) as s:
+        s.init(np.ones((ny, nx)), *[np.zeros((ny, nx))] * 2, np.ones((ny, nx)))
+        s.set_f(f)
+        s.step(1)
+        return f.astype(LD) - s.get_f()
+
+
 @pytest.mark.parametrize("log2n", [2, 3, 4, 5, 6, 8, 9, 10, 12])
 def test_line_derivative_error_by_kind_of_line(log2n):
     n, dt, d = 1 << log2n, 2.0 ** 60, D2V16()
@@ -82,30 +92,49 @@ def test_line_derivative_error_by_kind_of_line(log2n):
     plain = np.fft.irfft(1j * multiplier(n, np.float64) * np.fft.rfft(np.array(flat), axis=1), n, axis=1)[:, where]
     rms = lambda e: np.sqrt(np.sum(np.asarray(e, dtype=LD) ** 2, axis=1)).astype(float)
     bound = 2 * rms(plain - truth) + 12 * 2.0 ** -53 * rms(truth)
-    # a pair's bound is that of its two lines together: they share the integers' exponent
+    # a pair's bound is that of its two lines together: they share a complex line
     bound = np.hypot(bound[0::2], bound[1::2])
     got = []  # per axis and kind: its two lines' derivatives
-
-    def step(f):
-        ny, nx = f.shape[1:]
-        with lbm.Simulation(nx, ny, lbm.default_params(flags=FLAGS, dt=dt, tau=1.0, dx=1.0, dy=1.0)) as s:
-            s.init(np.ones((ny, nx)), *[np.zeros((ny, nx))] * 2, np.ones((ny, nx)))
-            s.set_f(f)
-            s.step(1)
-            return f.astype(LD) - s.get_f()
-
     for first in range(0, len(names), len(PAIRS)):  # rows
         f = np.ones((16, 4, n))
         for name, (a, b) in zip(names[first:], PAIRS):
             f[a], f[b] = by_kind[name][0][None, :], by_kind[name][1][None, :]
-        out = step(f)
+        out = difference(f, dt)
         got += [("rows", p, [out[i][1][where] / (dt * d.vx[i]) for i in PAIRS[p - first]])
                 for p in range(first, min(first + len(PAIRS), len(names)))]
     f = np.ones((16, n, 4))  # columns, the two lines in turn
     for p, i in enumerate(COLUMNS[:len(names)]):
         f[i] = np.stack([by_kind[names[p]][c & 1] for c in range(4)], axis=1)
-    out = step(f)
+    out = difference(f, dt)
     got += [("columns", p, [out[i][where, c] / (dt * d.vy[i]) for c in (0, 1)]) for p, i in enumerate(COLUMNS[:len(names)])]
     for axis, p, lines in got:
         err = np.hypot(*rms(np.asarray(lines, dtype=LD) - truth[2 * p:2 * p + 2]))
         assert err <= bound[p], (n, axis, names[p], err, bound[p])
+
+
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("log2n", [3, 6, 8, 10])
+def test_small_line_beside_a_large_one(log2n, axis):
+    """The two lines of a complex line have exponents of their own: one 1e-9 times the other (a dilute density
+    beside the temperature) keeps its accuracy. The bound is each line's own as above, and its partner's
+    at the same scale, which the transform may leave in it."""
+    n, dt, d = 1 << log2n, 2.0 ** 60, D2V16()
+    x = np.arange(n)
+    lines = np.array([1e-9 * (1 + 0.2 * np.sin(2 * np.pi * x / n)), 0.9 + 1e-3 * np.cos(2 * np.pi * x / n)])
+    where = np.arange(n) if n <= 512 else np.r_[:200]
+    truth = exact(lines, n, where)
+    plain = np.fft.irfft(1j * multiplier(n, np.float64) * np.fft.rfft(lines, axis=1), n, axis=1)[:, where]
+    rms = lambda e: np.sqrt(np.sum(np.asarray(e, dtype=LD) ** 2, axis=1)).astype(float)
+    own = 2 * rms(plain - truth) + 12 * 2.0 ** -53 * rms(truth)
+    top = np.abs(lines).max(axis=1)
+    bound = own + own[::-1] * top / top[::-1]
+    f = np.ones((16, 4, n))
+    if axis == 0:
+        f[0], f[2] = lines[0], lines[1]
+        out = difference(f, dt)
+        got = [out[0][1][where] / (dt * d.vx[0]), out[2][1][where] / (dt * d.vx[2])]
+    else:
+        f[1] = lines[[0, 1, 0, 1]]
+        out = difference(np.ascontiguousarray(np.swapaxes(f, 1, 2)), dt)
+        got = [out[1][where, c] / (dt * d.vy[1]) for c in (0, 1)]
+    assert np.all(rms(np.asarray(got) - truth) <= bound)
