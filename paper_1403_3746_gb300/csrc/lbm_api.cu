@@ -561,11 +561,20 @@ int capture_into(lbm_ctx *c, cudaStream_t s) {
 // steps does not pay (mixed 256^2 57.4 -> 55.6 us per step, five 128^2 as a batch 61.5 -> 59.8).
 constexpr int kManySteps = 8, kManyAfter = 32;
 
+// A graph is built in the middle of a run, when this or another thread may be capturing some other
+// stream: its calls on the library's own capture stream must not invalidate that capture.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // One step's launches as a CUDA graph: c->graph, or for a fused diagnostics request in slot
 // `slot` (>= 0) c->graph_diag[slot], whose first macro pass also writes the diagnostics partial
 // values into fpart[slot].
 // count > 1: that many steps, into c->graph_many.
 int build_step_graph(lbm_ctx *c, int slot = -1, int count = 1) {
+    RelaxedCapture relaxed;
     if (!c->cap) CU_TRY(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
     CU_TRY(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeRelaxed));
     c->fuse_capture = slot;
@@ -2073,6 +2082,7 @@ int lbm_batch_init(lbm_batch b, int k, const double *rho, const double *ux, cons
 // One graph per step: the groups' launches are parallel branches forked from and joined back
 // into the capture stream.
 static int build_batch_graph(lbm_batch b, int count) {
+    RelaxedCapture relaxed;
     const size_t G = b->groups.size();
     if (!b->cap) CU_TRY(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
     if (!b->fork) CU_TRY(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
