@@ -152,6 +152,7 @@ struct lbm_ctx {
     cudaStream_t cap = nullptr;
     cudaGraphExec_t graph = nullptr;
     cudaGraphExec_t graph_many = nullptr;  // kManySteps steps
+    bool many_failed = false;              // it could not be built: not tried again with these shapes
     long long graph_steps = 0;             // steps launched as graphs
 
     // per-launch timing
@@ -182,6 +183,7 @@ struct lbm_batch_ctx {
     cudaEvent_t fork = nullptr;
     cudaGraphExec_t graph = nullptr;
     cudaGraphExec_t graph_many = nullptr;        // kManySteps steps: the groups run them independently
+    bool many_failed = false;
     long long graph_steps = 0;                   // steps launched as graphs
     std::vector<long long> steps;                // per instance, since its lbm_batch_init
     // persistent form (kernels_batch.cu): one launch per step over all instances
@@ -555,11 +557,12 @@ int capture_into(lbm_ctx *c, cudaStream_t s) {
     return rc;
 }
 
-// Steps per launch of c->graph_many (c's own steps, or a batch's), and the steps a handle takes one by
-// one before that graph is built: a graph's launch costs 4.1 us against 0.7 to 1.2 us per kernel
-// within one, and building one of 64 kernels a fraction of a millisecond, which a handle of few
-// steps does not pay (mixed 256^2 57.4 -> 55.6 us per step, five 128^2 as a batch 61.5 -> 59.8).
-constexpr int kManySteps = 8, kManyAfter = 32;
+// Steps per launch of c->graph_many (c's own steps, or a batch's), the steps a handle takes one by
+// one before that graph is built, and the steps that must be left in the call in which they were
+// taken: a graph's launch costs 4.1 us against 0.7 to 1.2 us per kernel within one (mixed 256^2 57.4 ->
+// 55.6 us per step, five 128^2 as a batch 61.5 -> 59.8), and building one of 64 kernels 0.3 ms, which
+// some 160 steps pay back.
+constexpr int kManySteps = 8, kManyAfter = 32, kManyWorth = 256;
 
 // A graph is built in the middle of a run, when this or another thread may be capturing some other
 // stream: its calls on the library's own capture stream must not invalidate that capture.
@@ -568,6 +571,35 @@ struct RelaxedCapture {
     RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
     ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
+
+// n steps as graph launches on `s`: `one` of one step and, for a handle or batch that keeps stepping,
+// `many` of kManySteps; build(count) makes either, taken() counts them.
+template <class Build, class Taken>
+int run_graphs(int n, cudaStream_t s, cudaGraphExec_t &one, cudaGraphExec_t &many, bool &failed, long long &launched,
+               Build build, Taken taken) {
+    const bool kept = launched >= kManyAfter;  // the handle had its single steps before this call
+    while (n > 0) {
+        int count = 1;
+        if (n >= kManySteps && launched >= kManyAfter && !failed && (many || kept || n >= kManyWorth)) {
+            if (!many) {
+                const std::string before = g_last_error;
+                if (build(kManySteps) != LBM_OK) {  // one by one then
+                    failed = true;
+                    g_last_error = before;
+                    cudaGetLastError();
+                }
+            }
+            if (!failed) count = kManySteps;
+        }
+        if (count == 1 && !one)
+            if (const int rc = build(1)) return rc;
+        CU_TRY(cudaGraphLaunch(count == 1 ? one : many, s));
+        launched += count;
+        taken(count);
+        n -= count;
+    }
+    return LBM_OK;
+}
 
 // One step's launches as a CUDA graph: c->graph, or for a fused diagnostics request in slot
 // `slot` (>= 0) c->graph_diag[slot], whose first macro pass also writes the diagnostics partial
@@ -601,6 +633,7 @@ void drop_graphs(lbm_ctx *c) {
     c->graph = nullptr;
     if (c->graph_many) cudaGraphExecDestroy(c->graph_many);
     c->graph_many = nullptr;
+    c->many_failed = false;
     for (cudaGraphExec_t &g : c->graph_diag) {
         if (g) cudaGraphExecDestroy(g);
         g = nullptr;
@@ -1506,24 +1539,9 @@ int lbm_step(lbm_handle c, int n) {
         }
         return LBM_OK;
     }
-    // a handle that keeps stepping runs kManySteps steps per graph
-    while (n >= kManySteps && c->graph_steps >= kManyAfter) {
-        if (!c->graph_many && build_step_graph(c, -1, kManySteps)) break;  // one by one then
-        CU_TRY(cudaGraphLaunch(c->graph_many, c->stream));
-        c->steps += kManySteps;
-        c->graph_steps += kManySteps;
-        n -= kManySteps;
-    }
-    if (n > 0 && !c->graph) {
-        int rc = build_step_graph(c);
-        if (rc) return rc;
-    }
-    for (; n > 0; --n) {
-        CU_TRY(cudaGraphLaunch(c->graph, c->stream));
-        ++c->steps;
-        ++c->graph_steps;
-    }
-    return LBM_OK;
+    return run_graphs(
+        n, c->stream, c->graph, c->graph_many, c->many_failed, c->graph_steps,
+        [c](int count) { return build_step_graph(c, -1, count); }, [c](int count) { c->steps += count; });
 }
 
 int lbm_moments_device(lbm_handle c, double *rho, double *ux, double *uy, double *T) {
@@ -2061,6 +2079,7 @@ int lbm_batch_autotune(lbm_batch b) {
         cudaGraphExecDestroy(b->graph_many);
         b->graph_many = nullptr;
     }
+    b->many_failed = false;
     if (b->form == LBM_BATCH_PERSISTENT) return autotune_persistent(b);
     return LBM_OK;
 }
@@ -2302,22 +2321,12 @@ int lbm_batch_step(lbm_batch b, int n) {
         for (long long &s : b->steps) s += n;
         return LBM_OK;
     }
-    int left = n;
-    for (; left >= kManySteps && b->graph_steps >= kManyAfter; left -= kManySteps) {
-        if (!b->graph_many && build_batch_graph(b, kManySteps)) break;  // one by one then
-        CU_TRY(cudaGraphLaunch(b->graph_many, b->stream));
-        b->graph_steps += kManySteps;
-    }
-    if (left > 0 && !b->graph) {
-        int rc = build_batch_graph(b, 1);
-        if (rc) return rc;
-    }
-    for (; left > 0; --left) {
-        CU_TRY(cudaGraphLaunch(b->graph, b->stream));
-        ++b->graph_steps;
-    }
-    for (long long &s : b->steps) s += n;
-    return LBM_OK;
+    return run_graphs(
+        n, b->stream, b->graph, b->graph_many, b->many_failed, b->graph_steps,
+        [b](int count) { return build_batch_graph(b, count); },
+        [b](int count) {
+            for (long long &s : b->steps) s += count;
+        });
 }
 
 int lbm_batch_moments(lbm_batch b, int k, double *rho, double *ux, double *uy, double *T) {
