@@ -28,6 +28,13 @@ template <> struct Axis<double> {
 
 namespace reg {
 
+// What the float64 lines' reductions have room for: a line whose threads spread over 8 warps, and a
+// column tile of 16 lines (rows of 256 bytes); the launchers take no more.
+constexpr int kLineWarps = 8, kTileLines = 16;
+template <typename R> constexpr bool tile_fits(int lines, int threads) {
+    return sizeof(R) == 4 || (lines <= kTileLines && threads <= 32 * kLineWarps);
+}
+
 // st: distance between the threads of consecutive t (1: a line's threads are consecutive, the row
 // passes; L: the L lines of a column tile are interleaved, line index fastest)
 template <typename R, int LOG2N, bool PK, int CS = 1> struct Line : LineFFT<R, LOG2N, PK, CS> {
@@ -44,6 +51,9 @@ template <typename R, int LOG2N, bool PK, int CS = 1> struct Line : LineFFT<R, L
     template <class SYNC> static __device__ __forceinline__ void inverse(CT v[B::E], CT *buf, int t, const Axis<R> &ax, Scale) {
         B::template inverse<SYNC>(v, buf, t, ax.tw);
     }
+    // barriers only, of forward, and of multiply and inverse (see LineFFT)
+    template <class SYNC> static __device__ __forceinline__ void idle_forward(int) { B::template idle_forward<SYNC>(); }
+    template <class SYNC> static __device__ __forceinline__ void idle_inverse(int) { B::template idle_inverse<SYNC>(); }
 };
 
 template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineFFT<long long, LOG2N, false, CS> {
@@ -99,13 +109,13 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
         static_assert(SLOT + W <= kSlots, "scratch words");
         if constexpr (G == 1) return;
         const int tid = threadIdx.x, lane = tid & 31;
-        const int n = GL * st;  // threads over which the line's threads spread
+        const int n = GL * st;  // threads over which the line's threads spread (spans_warps: more than a warp's)
         const unsigned mask = n >= 32 ? 0xffffffffu : ((1u << n) - 1u) << (lane & ~(n - 1));
         for (int off = st; off < 32 && off < n; off <<= 1)
 #pragma unroll
             for (int k = 0; k < W; ++k) w[k] = op(k, w[k], __shfl_xor_sync(mask, w[k], off));
-        if (n > 32) {
-            // one entry per warp and line: a line spans at most 8 warps, and at most 16 lines of a tile share them
+        if (spans_warps(st)) {
+            // one entry per warp and line
             unsigned(*part)[kPart] = scratch();
             const int nw = n >> 5, wp = tid >> 5, l = tid & (st - 1);
             if (lane < st) {
@@ -116,18 +126,18 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
             const int w0 = wp & ~(nw - 1);
 #pragma unroll
             for (int k = 0; k < W; ++k) {
-                unsigned r[8];
+                unsigned r[kLineWarps];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) r[i] = i < nw ? part[SLOT + k][(w0 + i) * st + l] : 0u;
+                for (int i = 0; i < kLineWarps; ++i) r[i] = i < nw ? part[SLOT + k][(w0 + i) * st + l] : 0u;
 #pragma unroll
-                for (int d = 1; d < 8; d <<= 1)
+                for (int d = 1; d < kLineWarps; d <<= 1)
 #pragma unroll
-                    for (int i = 0; i + d < 8; i += 2 * d) r[i] = op(k, r[i], r[i + d]);
+                    for (int i = 0; i + d < kLineWarps; i += 2 * d) r[i] = op(k, r[i], r[i + d]);
                 w[k] = r[0];
             }
         }
         if constexpr (CS > 1) {  // the other CTAs' parts of the line, through distributed shared memory
-            __shared__ unsigned cpart[W][CS * 32];
+            __shared__ unsigned cpart[W][CS * kTileLines];
             const int l = tid & (st - 1);
             cluster_barrier();
             if (tid < st) {
@@ -135,7 +145,7 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
                 for (int r = 0; r < CS; ++r)
 #pragma unroll
                     for (int k = 0; k < W; ++k) {
-                        const uint32_t p = cluster_map(&cpart[k][cluster_rank() * 32 + l], r);
+                        const uint32_t p = cluster_map(&cpart[k][cluster_rank() * kTileLines + l], r);
                         asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(p), "r"(w[k]) : "memory");
                     }
             }
@@ -144,7 +154,7 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
             for (int k = 0; k < W; ++k) {
                 unsigned r[CS];
 #pragma unroll
-                for (int i = 0; i < CS; ++i) r[i] = cpart[k][i * 32 + l];
+                for (int i = 0; i < CS; ++i) r[i] = cpart[k][i * kTileLines + l];
 #pragma unroll
                 for (int d = 1; d < CS; d <<= 1)
 #pragma unroll
@@ -153,7 +163,8 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
             }
         }
     }
-    static constexpr int kPart = 128;
+    static __device__ __forceinline__ bool spans_warps(int st) { return GL * st > 32; }
+    static constexpr int kPart = kLineWarps * kTileLines;
     static __device__ __forceinline__ unsigned (*scratch())[kPart] {
         __shared__ unsigned part[kSlots][kPart];
         return part;
@@ -300,19 +311,19 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
         }
     }
 
-    // barriers only (see LineFFT), of forward and of multiply and inverse: the reductions of a line that
-    // spans warps add one each
-    template <class SYNC> static __device__ __forceinline__ void idle_forward() {
+    // barriers only, of forward, and of multiply and inverse (see LineFFT): those of the reductions of a
+    // line that spans warps as well
+    template <class SYNC> static __device__ __forceinline__ void idle_forward(int st) {
         static_assert(CS == 1, "float64 rows are not split over clusters");
-        if constexpr (GL > 32) {
+        if (spans_warps(st)) {
             SYNC::run();
             SYNC::run();
         }
         B::template idle_forward<SYNC>();
     }
-    template <class SYNC> static __device__ __forceinline__ void idle_inverse() {
+    template <class SYNC> static __device__ __forceinline__ void idle_inverse(int st) {
         static_assert(CS == 1, "float64 rows are not split over clusters");
-        if constexpr (GL > 32) SYNC::run();
+        if (spans_warps(st)) SYNC::run();
         B::template idle_inverse<SYNC>();
     }
 };

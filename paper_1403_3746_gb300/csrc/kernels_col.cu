@@ -55,6 +55,7 @@ template <typename R> static int jobs_acc(const ColArgs<R> &a, int njobs) {
 template <typename R, int LOG2N, int CS, bool ACC>
 static cudaError_t launch_col_cs_t(const ColArgs<R> &a, int njobs, size_t smem, cudaStream_t s) {
     using F = reg::Line<R, LOG2N, true, CS>;
+    if (!reg::tile_fits<R>(a.W / 2, (a.W / 2) * F::GL)) return cudaErrorInvalidValue;
     dim3 grid((a.nx / a.W) * CS, njobs, a.nb > 0 ? a.nb : 1);
     if constexpr (CS == 1) {
         cudaError_t e = allow_smem(col_deriv_kernel<R, LOG2N, ACC>);
@@ -231,7 +232,7 @@ template <typename R, int LOG2N, bool ACC>
 static cudaError_t launch_col_tma_t(const ColTmaArgs<R> &a, size_t smem, cudaStream_t s) {
     using F = reg::Line<R, LOG2N, true>;
     const int threads = (a.c.W / 2) * F::G;
-    if (threads > PassThreads<R>::value ||
+    if (threads > PassThreads<R>::value || !reg::tile_fits<R>(a.c.W / 2, threads) ||
         a.stage_bytes < (unsigned)((a.c.W / 2) * col_line_stride(LOG2N, sizeof(R), 1) * sizeof(typename F::CT)))
         return cudaErrorNotSupported;
     cudaError_t e = allow_smem(col_tma_kernel<R, LOG2N, ACC>);

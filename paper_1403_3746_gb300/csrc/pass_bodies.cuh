@@ -24,8 +24,8 @@ __device__ __forceinline__ void col_tile(const ColArgs<R> &a, int jobi, int z, i
     const int L = a.W >> 1;
     if constexpr (EXTRA) {
         if ((int)threadIdx.x >= L * F::GL) {
-            F::template idle_forward<reg::SyncCta>();
-            F::template idle_inverse<reg::SyncCta>();
+            F::template idle_forward<reg::SyncCta>(L);
+            F::template idle_inverse<reg::SyncCta>(L);
             return;
         }
     }
@@ -153,15 +153,15 @@ __device__ __forceinline__ void macro_rows(const MacroArgs<R> &a, int blk) {
     auto line_round = [&](int it) {
         if (!active) {  // the barriers of the line groups
             for (int k = 0; k < (SERIAL && it != 1 ? 2 : 1); ++k) {
-                if (it != 1) F::template idle_forward<reg::SyncCta>();
-                F::template idle_inverse<reg::SyncCta>();
+                if (it != 1) F::template idle_forward<reg::SyncCta>(1);
+                F::template idle_inverse<reg::SyncCta>(1);
                 if (it != 2) reg::cta_barrier();
             }
             return;
         }
         for (int kind = my_kind; kind <= (SERIAL && it != 1 ? 1 : my_kind); ++kind) {
             if (it == 1 && kind == 1) {
-                F::template idle_inverse<reg::SyncCta>();
+                F::template idle_inverse<reg::SyncCta>(1);
                 reg::cta_barrier();
                 continue;
             }
@@ -792,8 +792,8 @@ __device__ __forceinline__ void update_rows(const UpdateArgs<R> &a, const Update
                 if constexpr (CS == 1) reg::cta_barrier();  // (a split inverse ends with a cluster barrier)
                 F::store_natural(v, buf, t);
             } else {
-                F::template idle_forward<reg::SyncCta>();
-                F::template idle_inverse<reg::SyncCta>();
+                F::template idle_forward<reg::SyncCta>(1);
+                F::template idle_inverse<reg::SyncCta>(1);
                 if constexpr (CS == 1) reg::cta_barrier();
             }
         }
