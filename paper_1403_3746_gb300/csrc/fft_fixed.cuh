@@ -72,9 +72,9 @@ __host__ __device__ __forceinline__ int bal_hi(long long a) {
 // with a plain carry: three wide multiply-adds and two additions.
 constexpr unsigned long long kMidBias = 0x8000000080000000ULL;  // 2^63, and 2^31 to round
 constexpr unsigned long long kHighBias = 0ULL - 0x80000000ULL;
-// a b + c with 32-bit signed factors as one instruction (written as PTX: as a 64-bit product of
-// sign-extended factors it was compiled to an unsigned wide product and two corrections, 49% more
-// instructions in the whole column pass)
+// a b + c with 32-bit signed factors, written as PTX's signed wide multiply-add: with products of
+// 64-bit factors the column pass executed 49% more instructions (ncu's counter) and took 656 us per
+// 1024^2 step instead of 484
 __host__ __device__ __forceinline__ unsigned long long madw(int a, int b, unsigned long long c) {
 #ifdef __CUDA_ARCH__
     unsigned long long r;
