@@ -171,9 +171,6 @@ __device__ __forceinline__ void cta_barrier() { asm volatile("barrier.sync 0;" :
 struct SyncCta {
     static __device__ __forceinline__ void run() { cta_barrier(); }
 };
-struct SyncWarp {
-    static __device__ __forceinline__ void run() { __syncwarp(); }
-};
 
 // ---- thread-block clusters: a line split over CS CTAs of one cluster ----------------------
 // rank of this CTA in its cluster
@@ -198,9 +195,6 @@ __device__ __forceinline__ uint32_t cluster_map(const void *p, unsigned rank) {
 __device__ __forceinline__ void st_cluster(uint32_t a, float2 v) {
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
 }
-__device__ __forceinline__ void st_cluster(uint32_t a, double2 v) {
-    asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v.x), "d"(v.y) : "memory");
-}
 __device__ __forceinline__ void st_cluster(uint32_t a, longlong2 v) {
     asm volatile("st.shared::cluster.v2.b64 [%0], {%1, %2};" ::"r"(a), "l"(v.x), "l"(v.y) : "memory");
 }
@@ -209,9 +203,6 @@ __device__ __forceinline__ void ld_cluster(uint32_t a, float2 &v) {
 }
 __device__ __forceinline__ void ld_cluster(uint32_t a, longlong2 &v) {
     asm volatile("ld.shared::cluster.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a) : "memory");
-}
-__device__ __forceinline__ void ld_cluster(uint32_t a, double2 &v) {
-    asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
 }
 
 // Twiddle table of a line length n = 2^log2n: for each radix-16 pass P (span S = n / 16^P,
@@ -486,8 +477,7 @@ template <typename R, int LOG2N, bool PK = false, int CS = 1> struct LineFFT {
 
     // Forward DFT of a line held as v[e] = x[t + G e]; on return v[e] = X at digit-reversed
     // position E t + e. buf: this line's shared buffer of SMEM elements. Every thread of the
-    // block (SyncCta) or warp (SyncWarp) must call it; with a cluster split, every thread of
-    // the cluster.
+    // block must call it (or its idle form); with a cluster split, every thread of the cluster.
     template <class SYNC> static __device__ __forceinline__ void forward(CT v[E], CT *buf, int t,
                                                                         const CT *__restrict__ tw) {
         if constexpr (LOOPED) forward_loop<SYNC>(v, buf, t, tw);

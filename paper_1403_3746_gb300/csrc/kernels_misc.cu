@@ -288,10 +288,9 @@ cudaError_t launch_rho64(const float *f, double *r64, int nx, int ny, cudaStream
 
 template <int LOG2N> static cudaError_t launch_rho64_rows_n(double *r64, const Axis<double> &ax, int ny, cudaStream_t s) {
     using F = reg::Line<double, LOG2N, false>;
-    // about 128 threads per CTA: two CTAs' line buffers fit an SM at 1024 points
-    int lines = F::G < 128 ? 128 / F::G : 1;
-    while ((ny / 2) % lines) lines >>= 1;
-    const size_t smem = (size_t)lines * 2 * F::STRIDE * sizeof(double2);
+    static_assert(F::STRIDE == line_smem(LOG2N), "line buffers as rho64_row_smem counts them");
+    const int lines = rho64_row_pairs(LOG2N, ny);
+    const size_t smem = rho64_row_smem(LOG2N, ny);
     cudaError_t e = allow_smem(rho64_row_kernel<LOG2N>);
     if (e != cudaSuccess) return e;
     rho64_row_kernel<LOG2N><<<ny / (2 * lines), lines * F::G, smem, s>>>(r64, ax);

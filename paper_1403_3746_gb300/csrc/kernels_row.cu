@@ -78,38 +78,37 @@ template <typename R, int LOG2N> static cudaError_t launch_macro_n(const MacroAr
     const size_t need = (size_t)3 * a.rows * F::STRIDE * sizeof(typename F::CT);
     if (smem < need) return cudaErrorInvalidValue;
     const int threads = macro_cta_threads(a.rows, LOG2N, sizeof(R), a.serial);
-    if constexpr (sizeof(R) == 8 && LOG2N == 12) {  // the only shape that needs the serial form
-        if (a.serial) {
-            if (a.r64) return cudaErrorInvalidValue;
-            cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, true, false>);
-            if (e != cudaSuccess) return e;
-            macro_row_kernel<R, LOG2N, true, false><<<a.ny / a.rows, threads, smem, s>>>(a);
-            return cudaGetLastError();
+    if constexpr (sizeof(R) == 8 && LOG2N == 12) {  // the shape that needs the serial form, and takes no other
+        if (!a.serial || a.r64) return cudaErrorInvalidValue;
+        cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, true, false>);
+        if (e != cudaSuccess) return e;
+        macro_row_kernel<R, LOG2N, true, false><<<a.ny / a.rows, threads, smem, s>>>(a);
+        return cudaGetLastError();
+    } else {
+        if (a.serial) return cudaErrorInvalidValue;
+        if (a.diag_partial && (sizeof(R) != 4 || a.r64)) return cudaErrorInvalidValue;
+        if constexpr (sizeof(R) == 4) {
+            if (a.diag_partial) {  // the diagnostics of the input state fused in
+                cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, false, true>);
+                if (e != cudaSuccess) return e;
+                macro_row_kernel<R, LOG2N, false, false, true><<<a.ny / a.rows, threads, smem, s>>>(a);
+                return cudaGetLastError();
+            }
         }
-    }
-    if (a.serial) return cudaErrorInvalidValue;
-    if (a.diag_partial && (sizeof(R) != 4 || a.r64)) return cudaErrorInvalidValue;
-    if constexpr (sizeof(R) == 4) {
-        if (a.diag_partial) {  // the diagnostics of the input state fused in
-            cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, false, true>);
-            if (e != cudaSuccess) return e;
-            macro_row_kernel<R, LOG2N, false, false, true><<<a.ny / a.rows, threads, smem, s>>>(a);
-            return cudaGetLastError();
+        if constexpr (sizeof(R) == 4) {  // the float64 density chain (LBM_MIXED_RHO64)
+            if (a.r64) {
+                cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, true>);
+                if (e != cudaSuccess) return e;
+                macro_row_kernel<R, LOG2N, false, true><<<a.ny / a.rows, threads, smem, s>>>(a);
+                return cudaGetLastError();
+            }
         }
+        if (a.r64) return cudaErrorInvalidValue;
+        cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, false>);
+        if (e != cudaSuccess) return e;
+        macro_row_kernel<R, LOG2N, false, false><<<a.ny / a.rows, threads, smem, s>>>(a);
+        return cudaGetLastError();
     }
-    if constexpr (sizeof(R) == 4) {  // the float64 density chain (LBM_MIXED_RHO64)
-        if (a.r64) {
-            cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, true>);
-            if (e != cudaSuccess) return e;
-            macro_row_kernel<R, LOG2N, false, true><<<a.ny / a.rows, threads, smem, s>>>(a);
-            return cudaGetLastError();
-        }
-    }
-    if (a.r64) return cudaErrorInvalidValue;
-    cudaError_t e = allow_smem(macro_row_kernel<R, LOG2N, false, false>);
-    if (e != cudaSuccess) return e;
-    macro_row_kernel<R, LOG2N, false, false><<<a.ny / a.rows, threads, smem, s>>>(a);
-    return cudaGetLastError();
 }
 
 template <typename R> cudaError_t launch_update(const UpdateArgs<R> &a, size_t smem, cudaStream_t s) {

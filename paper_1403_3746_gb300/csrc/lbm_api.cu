@@ -933,7 +933,7 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
         std::max(std::max(c->geo.upd_smem, c->geo.macro_smem), std::max(c->geo.col_smem, c->geo.rowd_smem));  // flux = col
     if (c->rho64) {  // the density chain's float64 column and row transforms
         pass_geometry(nx, ny, 8, &c->geo64, nb);
-        need = std::max(need, std::max(c->geo64.col_smem, c->geo64.rowd_smem));
+        need = std::max(need, std::max(c->geo64.col_smem, rho64_row_smem(c->lx, nb * ny)));
     }
     if (need > (size_t)smem_optin) {
         delete c;

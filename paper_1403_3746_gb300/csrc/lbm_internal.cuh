@@ -272,7 +272,14 @@ template <typename R> struct MacroArgs {
 enum Rho64Field { R64_RHO, R64_RX, R64_RXX, R64_RY, R64_RYY, NR64 };
 // rho in float64 as the sum of the 16 stored distributions of each node (f: [ny][16][nx])
 cudaError_t launch_rho64(const float *f, double *r64, int nx, int ny, cudaStream_t s);
-// d_x rho and d_xx rho of all ny rows (an even number) of the density chain
+// d_x rho and d_xx rho of all ny rows (an even number) of the density chain: row pairs per CTA, about 128
+// threads (two CTAs' line buffers fit an SM at 1024 points), and its shared memory, two buffers per pair
+constexpr int rho64_row_pairs(int log2n, int ny) {
+    int n = line_G(log2n) < 128 ? 128 / line_G(log2n) : 1;
+    while ((ny / 2) % n) n >>= 1;
+    return n;
+}
+constexpr size_t rho64_row_smem(int log2n, int ny) { return (size_t)rho64_row_pairs(log2n, ny) * 2 * line_smem(log2n) * sizeof(double2); }
 cudaError_t launch_rho64_rows(double *r64, const Axis<double> &ax, int ny, cudaStream_t s);
 // initial-field validity: the lowest failing node index into *bad (untouched if none fails)
 cudaError_t launch_check_init(const double *rho, const double *ux, const double *uy, const double *T, long long n,
