@@ -277,7 +277,8 @@ int lbm_set_pass_kinds(lbm_handle h, const int kinds[3]);
 
 /* Fault injection for tests (no counterpart in the paper). Every device-side wait of the
  * library (the TMA column pass waiting for its copies) is bounded by `wait_cycles` clock
- * cycles (<= 0: the default, about one second); a wait that runs out makes its kernel record
+ * cycles of polling (<= 0: the default, about one second; a stretch in which the GPU ran another
+ * process instead counts for 8 ms at most); a wait that runs out makes its kernel record
  * the failure in the handle's device error word and return, and the next synchronising call
  * (lbm_synchronize, lbm_moments, lbm_get_f, lbm_get_state, lbm_diagnostics) returns
  * LBM_ERR_TIMEOUT once. LBM_FAULT_STARVE_COPIES makes the TMA column pass arm its barriers

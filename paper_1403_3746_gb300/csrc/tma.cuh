@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "wait_budget.cuh"
+
 namespace lbm {
 namespace tma {
 
@@ -55,11 +57,12 @@ __device__ __forceinline__ bool bar_try_wait(uint64_t *bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// waits for the barrier's phase `parity` to complete; false if `budget` clock cycles pass first
+// waits for the barrier's phase `parity` to complete; false if `budget` clock cycles of polling pass
+// first (wait_budget.cuh)
 __device__ __forceinline__ bool bar_wait_bounded(uint64_t *bar, uint32_t parity, long long budget) {
-    const long long t0 = clock64();
+    WaitBudget wait(clock64(), budget);
     while (!bar_try_wait(bar, parity)) {
-        if (clock64() - t0 > budget) return false;
+        if (wait.spent(clock64())) return false;
     }
     return true;
 }
