@@ -1121,7 +1121,14 @@ int moments_host(lbm_ctx *c, int k, double *rho, double *ux, double *uy, double 
     double err = 0.0;
     int rc = moments_to_device(c, k, dev, st + 4 * n);
     if (rc) return rc;
-    if (4 * n <= kSmallRead) {
+    // (a target that is device memory goes by the copies, which answer for it)
+    auto on_device = [](const void *p) {
+        cudaPointerAttributes a;
+        const bool known = p && cudaPointerGetAttributes(&a, p) == cudaSuccess;
+        if (p && !known) cudaGetLastError();
+        return known && a.type == cudaMemoryTypeDevice;
+    };
+    if (4 * n <= kSmallRead && !on_device(rho) && !on_device(ux) && !on_device(uy) && !on_device(T)) {
         std::vector<double> buf(4 * n + 1);
         CU_TRY(cudaMemcpyAsync(buf.data(), st, buf.size() * 8, cudaMemcpyDeviceToHost, c->stream));
         CU_TRY(cudaStreamSynchronize(c->stream));
