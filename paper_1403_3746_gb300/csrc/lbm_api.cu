@@ -163,7 +163,8 @@ struct lbm_ctx {
 
     // Columns of two points have only the mean and the Nyquist index, whose multipliers are zero: every
     // y-derivative of a step is zero, as the fields that hold them are from the start, and no column
-    // pass runs (quasi-one-dimensional runs of two rows: 8 kernels per step -> 4, 512 x 2 mixed 40.4 -> 31.6 us)
+    // pass runs (quasi-one-dimensional runs of two rows: 8 kernels per step -> 4, 512 x 2 mixed 40.4 -> 31.6
+    // us). The rows do not depend on one another, so a row that is no longer finite leaves the other as it is.
     bool y_derivatives_vanish() const { return ny == 2; }
     bool all_initialized() const {
         for (char v : initialized)
@@ -2520,12 +2521,12 @@ void pass_geometry(int nx, int ny, size_t esize, Geometry *g, int nb) {
     if (r0 < 1) r0 = 1;
     if (r0 > ny) r0 = ny;
     // float64 nodes are bound by each SM's own float64 unit: fewer rows per CTA until there is a CTA
-    // for each of the 152 SMs (64^2: 8 rows -> 1, update pass 67 -> 35 us per launch)
+    // for each SM (64^2: 8 rows -> 1, update pass 67 -> 35 us per launch)
     const long long rows = (long long)ny * nb;
-    while (esize == 8 && r0 > 1 && rows / r0 < 152) r0 >>= 1;
+    while (esize == 8 && r0 > 1 && rows / r0 < kSms) r0 >>= 1;
     int r = r0;
     // float32 update pass of small grids: until two CTAs per SM (128^2 step 48.4 -> 46.3 us)
-    while (esize == 4 && r > 1 && rows / r < 304) r >>= 1;
+    while (esize == 4 && r > 1 && rows / r < 2 * kSms) r >>= 1;
     while (r > 1 && 6 * r * SM > 200 * 1024) r >>= 1;  // update: 6 line buffers per row
     g->rows_upd = r;
     g->upd_smem = 6 * (size_t)r * SM;
@@ -2547,7 +2548,7 @@ void pass_geometry(int nx, int ny, size_t esize, Geometry *g, int nb) {
     const int mact = macro_threads(esize, lx);
     // float64 macro pass: the lines of up to 128 threads per CTA, so that its warps share the fetch of
     // the transforms' code, while there are 128 CTAs (512^2 step 780 -> 724 us, 128 x 256 181 -> 177,
-    // 256 x 2048 1250 -> 1174)
+    // 256 x 2048 1250 -> 1174; with a CTA for each of the 152 SMs 256 rows would go by one instead of two)
     if (esize == 8) {
         r = 1;
         while (2 * r <= ny && 4 * r * G <= 128 && rows / (2 * r) >= 128) r *= 2;

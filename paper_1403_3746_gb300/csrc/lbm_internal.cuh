@@ -185,6 +185,8 @@ struct Geometry {
     int col_kind = 0;           // column pass: LBM_COL_DIRECT, LBM_COL_TMA, LBM_COL_LOOKAHEAD or LBM_COL_TMA1 (width colW)
     int flux_kind = 0;          // flux column pass: the same choice (width fluxW)
 };
+// SMs of a GB300, which the rules are written for (a constant, so that a plan is the same on any host)
+constexpr int kSms = 152;
 // nb: instances stacked along y
 void pass_geometry(int nx, int ny, size_t esize, Geometry *g, int nb = 1);
 
