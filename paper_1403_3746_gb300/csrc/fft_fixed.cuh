@@ -17,7 +17,8 @@
 //
 // The spectrum is shifted up before it meets the multiplier, as far as its largest entry with a
 // non-zero multiplier allows, and the products again, until their summed magnitudes fill 2^63: the
-// mean and the low indices, whose multipliers are small, would otherwise leave the rest few bits.
+// mean and the low indices, whose multipliers are small, would otherwise leave the rest few bits. (Up
+// to 256 points the sum of the points themselves is enough, and cheaper.)
 // Where the sum is larger than that without a shift, no sum overflows all the same: the products'
 // 2-norm is at most N^(1/2) / 4^(T + 1) times the line's (T twiddled passes, the factor 1/4 of the
 // product), and a sum of P of them at most sqrt(P) times that (Cauchy-Schwarz); line_bits keeps it
@@ -34,8 +35,8 @@
 // Measured against the float64 transforms (1024^2): column pass 1225 -> 254 us per launch of 17
 // fields, flux pass 330 -> 83; float64 step 8.31 -> 2.44 ms with the node loops and launch shapes.
 // The passes wait for instructions and on latency, both integer pipes about half busy at 16 warps per
-// SM. The two exponents, the mean, the sums and the two shifts are 4 to 7% of a step (1024^2 2.31 -> 2.44
-// ms, 128 x 256 180 -> 193 us, 64^2 unchanged); without them the errors were 2 to 14 times float64's for
+// SM. The two exponents, the mean, the sums and the two shifts are 3 to 6% of a step (1024^2 2.31 -> 2.44
+// ms, 128 x 256 180 -> 191 us, 64^2 unchanged); without them the errors were 2 to 14 times float64's for
 // sharp levels close to one another, up to 25 times for single points on a constant, from 512 points
 // on, lines of 4 points constant to 10^-8 kept 9 digits of their derivative, and a line 10^-9 times its
 // partner 8.

@@ -91,10 +91,9 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
         B::store_natural(u, reinterpret_cast<longlong2 *>(buf), t);
     }
 
-    // Lines of up to 64 points take as many bits as the largest magnitude allows and keep their mean, and
-    // the multiplier's shift is that of the sum of the points: their errors are at most the float64
-    // transform's as it is, and their passes wait for instructions (64^2 float64 step 155 us, 167 with the
-    // general form).
+    // Lines of up to 64 points take as many bits as the largest magnitude allows and keep their mean: their
+    // errors are at most the float64 transform's as it is, and their passes wait for instructions (64^2
+    // float64 step 155 us, 167 with the general form).
     static constexpr bool kShort = LOG2N <= 6;
 
     static __device__ __forceinline__ long long shl(long long a, int n) { return (long long)((unsigned long long)a << n); }
@@ -243,7 +242,7 @@ template <int LOG2N, bool PK, int CS> struct Line<double, LOG2N, PK, CS> : LineF
             const int lz = fixed::clz64(sum);
             pre = max(lz - 8, 0);
             post = min(max(lz - 6, 0), 2);
-        } else if constexpr (kShort) {  // the points' sum in units of 2^40
+        } else if constexpr (LOG2N <= 8) {  // the points' sum in units of 2^40 (enough up to 256 points)
             unsigned r[1] = {2 * E};
 #pragma unroll
             for (int e = 0; e < E; ++e) {
