@@ -60,7 +60,8 @@ def peaks():
 # host orchestration (lbm_api.cu, lbm_noalloc.cu) is not part of it, and the launch shapes a
 # profile was taken with are checked separately
 DEVICE_SOURCES = ("fft_fixed.cuh", "fft_line.cuh", "fft_reg.cuh", "kernels_batch.cu", "kernels_col.cu",
-                  "kernels_misc.cu", "kernels_row.cu", "kernels_sf.cu", "lbm_internal.cuh", "pass_bodies.cuh", "tma.cuh")
+                  "kernels_misc.cu", "kernels_row.cu", "kernels_sf.cu", "lbm_internal.cuh", "pass_bodies.cuh", "tma.cuh",
+                  "wait_budget.cuh")
 
 
 def source_digest():
