@@ -85,6 +85,41 @@ bool moment_inverse(double eta0, double out[256]) {
     return true;
 }
 
+// The coefficients of f_i^eq / rho of each speed group (UpdateConst<double>), from the row of M^-1 (w[j]: of
+// moment j) of its first velocity, (v, 0) or (v, v), collected by powers of T, u^2 and d. They are the same in
+// every step and node, so their rounding adds up: each is rounded once, from rows of M^-1 with one Newton step
+// on the float64 inverse (residual in double-double). Collected in float64 from the inverse as it is they were
+// off by up to 7 2^-53 and took 4.5e-16 of the energy and 3.3e-16 of the mass per stage at rest, mean over T =
+// 0.8 .. 1, where these take 2e-17 and 3e-17 (the full product M^-1 m^eq: 2.3e-16 and 2.2e-16).
+void group_coefficients(double eta0, double b, const double minv[256], double out[4][10]) {
+    double rows[16][16];
+    moment_rows(eta0, rows);
+    for (int g = 0; g < 4; ++g) {
+        const double *x = minv + 4 * g * 16;
+        double r[16];  // e - x M
+        for (int i = 0; i < 16; ++i) {
+            double hi = i == 4 * g ? 1.0 : 0.0, lo = 0.0;
+            for (int j = 0; j < 16; ++j) {
+                const double p = -x[j] * rows[j][i], e = std::fma(-x[j], rows[j][i], -p), t = hi + p, z = t - hi;
+                lo += ((hi - (t - z)) + (p - z)) + e;
+                hi = t;
+            }
+            r[i] = hi + lo;
+        }
+        long double w[16];
+        for (int j = 0; j < 16; ++j) {
+            double d = 0.0;
+            for (int i = 0; i < 16; ++i) d = std::fma(r[i], minv[i * 16 + j], d);
+            w[j] = (long double)x[j] + d;
+        }
+        const long double bl = b, s2 = (w[4] + w[6]) / 2, s4 = (w[13] + w[15]) / 2;
+        const long double d2 = g < 2 ? (w[4] - w[6]) / 2 : w[5], d4 = g < 2 ? (w[13] - w[15]) / 2 : w[14];
+        const long double o[10] = {w[0], w[3] * bl + 2 * s2, w[3] + s2, s4, d2, d4,
+                                   w[1], w[7] * (bl + 2) + 3 * w[9] + w[11], w[7] + (w[9] + w[11]) / 2, (w[9] - w[11]) / 2};
+        for (int q = 0; q < 10; ++q) out[g][q] = (double)o[q];
+    }
+}
+
 }  // namespace
 
 struct lbm_ctx {
@@ -141,6 +176,7 @@ struct lbm_ctx {
     long long *kfx = nullptr, *kfy = nullptr;  // solution filter W(m) / N per axis (params filter_alpha > 0)
     float *kfx32 = nullptr, *kfy32 = nullptr;
     double minv[256];
+    double group_coef[4][10];  // float64 update pass (group_coefficients)
 
     Geometry geo;    // launch geometry
     Geometry geo64;  // float64 launch geometry of the density chain's transforms (rho64 only)
@@ -345,8 +381,6 @@ void fill_const(const lbm_ctx *c, UpdateConst<float> &k) {
     }
     for (int j = 0; j < 256; ++j) k.minv[j] = (float)c->minv[j];
 }
-// the coefficients of a speed group: the means over its four velocities' images of the entries of
-// M^-1 (w[j]: of moment j), then collected by powers of T, u^2 and d
 void fill_const(const lbm_ctx *c, UpdateConst<double> &k) {
     const double b = c->p.b;
     k.ib = 1.0 / b;
@@ -355,31 +389,7 @@ void fill_const(const lbm_ctx *c, UpdateConst<double> &k) {
     k.b6 = b + 6.0;
     for (int g = 0; g < 4; ++g) {
         k.psi[g] = vel_sq(4 * g) + (g == 0 ? c->p.eta0 * c->p.eta0 : 0.0);
-        double one = 0, en = 0, s2 = 0, s4 = 0, d2 = 0, d4 = 0, j = 0, pj = 0, aaa = 0, abb = 0;
-        for (int i = 4 * g; i < 4 * g + 4; ++i) {
-            const double *w = c->minv + i * 16;
-            const double sx = vel_x(i) > 0 ? 1.0 : vel_x(i) < 0 ? -1.0 : 0.0, sy = vel_y(i) > 0 ? 1.0 : vel_y(i) < 0 ? -1.0 : 0.0;
-            one += 0.25 * w[0];
-            en += 0.25 * w[3];
-            s2 += 0.125 * (w[4] + w[6]);
-            s4 += 0.125 * (w[13] + w[15]);
-            if (g < 2) {
-                const double s = sx != 0 ? 1.0 : -1.0;
-                d2 += 0.125 * s * (w[4] - w[6]);
-                d4 += 0.125 * s * (w[13] - w[15]);
-            } else {
-                d2 += 0.25 * sx * sy * w[5];
-                d4 += 0.25 * sx * sy * w[14];
-            }
-            const double wt = g < 2 ? 0.25 : 0.125;  // axis groups: each velocity sees one axis
-            j += wt * (sx * w[1] + sy * w[2]);
-            pj += wt * (sx * w[7] + sy * w[8]);
-            aaa += wt * (sx * w[9] + sy * w[12]);
-            abb += wt * (sx * w[11] + sy * w[10]);
-        }
-        const double o[10] = {one, en * b + 2.0 * s2, en + s2, s4, d2, d4,
-                              j, pj * (b + 2.0) + 3.0 * aaa + abb, pj + 0.5 * (aaa + abb), 0.5 * (aaa - abb)};
-        for (int q = 0; q < 10; ++q) k.c[g][q] = o[q];
+        for (int q = 0; q < 10; ++q) k.c[g][q] = c->group_coef[g][q];
     }
 }
 template <typename R> UpdateArgs<R> update_args(const lbm_ctx *c, int stage, int rows_per_cta) {
@@ -925,6 +935,7 @@ int create_ctx(int nx, int ny, int nb, const lbm_params *params, cudaStream_t st
         delete c;
         return fail(LBM_ERR_ARG, "moment matrix is singular for eta0=%g", params->eta0);
     }
+    if (!c->mixed) group_coefficients(params->eta0, params->b, c->minv, c->group_coef);
 
     // launch geometry
     int smem_optin = 0;
